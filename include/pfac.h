@@ -229,8 +229,9 @@ typedef struct {
                                   leaves), merged-trie indirection and side
                                   table */
     uint64_t index_bytes;      /* prefix nodes of every depth held (bitmaps,
-                                  counts, entries, child masks, prefix bytes)
-                                  and the gram filter; both layouts */
+                                  counts, entries, child masks, prefix bytes),
+                                  the gram filter and the window filter; both
+                                  layouts */
     uint64_t other_bytes;      /* patterns kept for verification (truncated
                                   tables) */
     uint32_t record_bytes;     /* bytes per node record (4, 8, 16 or 48; 0 for
@@ -272,6 +273,11 @@ int pfac_workspace_bytes(const pfac_table *t, uint64_t n_bytes, uint32_t n_segme
  * pfac_match_plan - the scan configuration a pfac_match call with these
  * options would use (no device work).  Library extension: the paper has no
  * counterpart.  Fields are 0 for the uncompressed layout except smem_bytes.
+ * Where the options leave every choice to the library, the table has no tuned
+ * choice and its pattern set makes a window filter that pays (a filter over
+ * short windows of the text, every S-th position looked up; built with the
+ * table), the scan pass runs over that filter; the fields then describe the
+ * plan that runs without it and whose emit pass the call uses.
  */
 typedef struct {
     uint32_t variant;        /* 1 or 2, as pfac_match_opts.variant */

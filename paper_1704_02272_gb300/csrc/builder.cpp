@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "window.h"
 
 namespace pfac {
 
@@ -586,6 +587,19 @@ extern "C" int pfac_build(const uint8_t *const *patterns, const uint32_t *length
             }
         }
         const uint64_t sz_G = Gv.size() * 4;
+        // ---- window filter (see table.h): plain tries, both layouts
+        WindowFilter wf;
+        if (!dag && match_density * 512.0 <= 8.0) {
+            std::vector<WinPat> wp(n_patterns);
+            for (uint32_t i = 0; i < n_patterns; i++) wp[i] = WinPat{pats[order[i]].p, len_at(i)};
+            // the deepest prefix bitmap of at most 64 KiB
+            double dens_f = 1.0;
+            for (uint32_t k = kmin; k <= kmax; k++)
+                if ((1ull << (k * bps)) <= 8ull * 65536)
+                    dens_f = (double)n_ent[k] / (double)(1ull << (k * bps));
+            build_window_filter(wp, sigma, bps, std::min(dens_f, 1.0), &wf);
+        }
+        const uint64_t sz_H = wf.H.size() * 4;
         // truncated tables keep the patterns for verification
         std::vector<uint32_t> pat_off;
         std::vector<uint8_t> pat_bytes;
@@ -754,6 +768,7 @@ extern "C" int pfac_build(const uint8_t *const *patterns, const uint32_t *length
             o_B[k] = place(sz_B[k]);
         }
         const uint64_t o_G = place(sz_G);
+        const uint64_t o_H = place(sz_H);
         const uint64_t o_po = place(sz_po), o_pb = place(sz_pb);
         uint64_t o_stt = place(sz_stt), o_dfin = place(sz_dfin);
         const uint64_t blob = std::max<uint64_t>(off, 256);
@@ -780,6 +795,7 @@ extern "C" int pfac_build(const uint8_t *const *patterns, const uint32_t *length
             put(o_B[k], Bv[k].data(), sz_B[k]);
         }
         put(o_G, Gv.data(), sz_G);
+        put(o_H, wf.H.data(), sz_H);
         put(o_po, pat_off.data(), sz_po);
         put(o_pb, pat_bytes.data(), sz_pb);
         if (dense) {
@@ -870,6 +886,15 @@ extern "C" int pfac_build(const uint8_t *const *patterns, const uint32_t *length
         dv.g_len = g_len;
         dv.g_bits = g_bits;
         dv.g_set = g_set;
+        dv.H = sz_H ? (const uint32_t *)(B + o_H) : nullptr;
+        dv.w_words = wf.words;
+        dv.w_rep = wf.rep;
+        dv.w_stride = wf.stride;
+        dv.w_nb = wf.nb;
+        dv.w_gw = wf.gw;
+        dv.w_glen = wf.glen;
+        dv.w_packed = wf.packed;
+        dv.w_short = wf.shorts;
         dv.stt = dense ? (const uint32_t *)(B + o_stt) : nullptr;
         dv.dfin = dense ? (const uint32_t *)(B + o_dfin) : nullptr;
         t->kmax = kmax;
@@ -898,7 +923,7 @@ extern "C" int pfac_build(const uint8_t *const *patterns, const uint32_t *length
         I.merged_trie_nodes = dag ? (uint64_t)n_upper + canon_rep.size() : 0;
         I.side_entries = side_n;
         I.trie_bytes = sz_rec + sz_fin + sz_fbc + sz_fv + sz_leaf + sz_pool + sz_ind + sz_sk + sz_sv;
-        I.index_bytes = sz_G;
+        I.index_bytes = sz_G + sz_H;
         for (uint32_t k = kmin; k <= kmax; k++)
             I.index_bytes += sz_F[k] + sz_C[k] + sz_E[k] + sz_M[k] + sz_B[k];
         // the dense layout's transition table and outputs are its trie

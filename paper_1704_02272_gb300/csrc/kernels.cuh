@@ -119,6 +119,16 @@ struct MatchParams {
     uint32_t defer_cap;
     uint32_t dbatch_cap;
     uint2 *dbatch;
+    // window kernel: the entry buffer (position << 24 | prefix index), the
+    // filter's split of shared memory and hash, the prefix bitmap of depth
+    // wf_k its candidates are tested against (wf_words of it in shared memory)
+    uint64_t *wbuf;
+    uint32_t wbuf_cap;
+    uint32_t w_words, w_rep, w_gm, w_glen;
+    uint32_t w_badmask;   // byte bits outside the symbol range, where they matter to the filter
+    const uint32_t *wf;
+    uint32_t wf_words, wf_k;
+    uint32_t unordered;  // a unit's records are in no order (the expansion sorts them)
 };
 
 constexpr uint32_t UNIT_NONE = 0xFFFFFFFFu;

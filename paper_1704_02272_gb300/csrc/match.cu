@@ -9,7 +9,7 @@
 #include <mutex>
 
 #include "internal.h"
-#include "kernels_r.cuh"
+#include "kernels_w.cuh"
 
 namespace pfac {
 
@@ -32,6 +32,12 @@ void *scan_kernel_r2_g1_f(int rep, int nw);
 void *scan_kernel_r2_g1_fe(int rep, int nw);
 
 void *resolve_kernel(int w);
+void *wresolve_kernel(int w);
+void *scan_kernel_w1(bool packed, uint32_t nb, bool g5, int tb);
+void *scan_kernel_w2(bool packed, uint32_t nb, bool g5, int tb);
+void *scan_kernel_w4(bool packed, uint32_t nb, bool g5, int tb);
+void *scan_kernel_w8(bool packed, uint32_t nb, bool g5, int tb);
+void *scan_kernel_w16(bool packed, uint32_t nb, bool g5, int tb);
 void *scan_kernel_r8_d0(int rep, int var, int nw);
 void *scan_kernel_r8_d1(int rep, int var, int nw);
 void *scan_kernel_r2_d0(int rep, int var, int nw);
@@ -52,6 +58,19 @@ static void *scan_kernel_r(uint32_t bps, uint32_t w, int rep, bool gram, int var
     if (bps != 8) return nullptr;
     if (gram) return var == VAR_FE ? scan_kernel_r8_g1_fe(rep, nw) : scan_kernel_r8_g1_f(rep, nw);
     return var == VAR_FE ? scan_kernel_r8_g0_fe(rep, nw) : scan_kernel_r8_g0_f(rep, nw);
+}
+
+// the window kernel for a table's filter
+static void *scan_kernel_w(const DevTable &T, int tb) {
+    const bool packed = T.w_packed != 0, g5 = !packed && T.w_gw == 5;
+    switch (T.w_stride) {
+        case 1: return scan_kernel_w1(packed, T.w_nb, g5, tb);
+        case 2: return scan_kernel_w2(packed, T.w_nb, g5, tb);
+        case 4: return scan_kernel_w4(packed, T.w_nb, g5, tb);
+        case 8: return scan_kernel_w8(packed, T.w_nb, g5, tb);
+        case 16: return scan_kernel_w16(packed, T.w_nb, g5, tb);
+        default: return nullptr;
+    }
 }
 
 constexpr int CHUNK = 1024;      // tiles per chunk of the key-count scan
@@ -219,72 +238,102 @@ __global__ void __launch_bounds__(RT) k_offsets(const MatchParams P) {
     }
 }
 
-// Writes the keys of every tile whose records were kept; the last CTA
+// Writes the keys of every unit whose records were kept; the last CTA
 // publishes the call's status.
-constexpr uint32_t EXPAND_THREAD_MAX = 32;  // records a single thread expands
-__global__ void __launch_bounds__(256) k_expand(const MatchParams P) {
-    __shared__ bool last;
-    // one thread per unit: most units hold a few records or none, so the
-    // units' loads are issued side by side rather than one unit per warp
-    const uint64_t nthr = (uint64_t)gridDim.x * blockDim.x;
-    const uint32_t *pool = P.T.pool;
-    for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < P.n_tiles; t += nthr) {
-        const uint32_t m = P.tile_m[t];
-        if (m == 0 || m > P.unit_cap || m > EXPAND_THREAD_MAX) continue;
-        uint64_t o = P.key_off[t];
-        const uint64_t *rr = P.recs + t * P.unit_cap;
-        const uint64_t tile_start = t << P.unit_shift;
-        for (uint32_t i = 0; i < m; i++) {
-            const uint64_t r = rr[i];
-            const uint32_t L = fin_len_c(P, (uint32_t)r);
-            const uint32_t *ids = fin_ids_c(P, (uint32_t)r);
-            const uint64_t pk = (P.pos_base + tile_start + (r >> 32)) << PFAC_ID_BITS;
-            for (uint32_t e = 0; e < L; e++, o++)
-                if (o < P.cap) P.out[o] = pk | __ldg(ids + e);
-        }
-    }
-    // units with more records (record space for every position): a whole
-    // warp per unit, 32 records at a time, each lane's keys placed by a warp
-    // scan of the records' key counts
-    if (P.unit_cap > EXPAND_THREAD_MAX) {
-        const uint32_t lane = threadIdx.x & 31;
-        const uint64_t gwarp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-        const uint64_t nwarps = nthr >> 5;
-        for (uint64_t t0 = gwarp * 32; t0 < P.n_tiles; t0 += nwarps * 32) {
-            const uint64_t tl = t0 + lane;
-            const uint32_t ml = tl < P.n_tiles ? P.tile_m[tl] : 0u;
-            uint32_t dense = __ballot_sync(0xFFFFFFFFu, ml > EXPAND_THREAD_MAX && ml <= P.unit_cap);
-            while (dense) {
-                const uint32_t j = __ffs(dense) - 1;
-                dense &= dense - 1;
-                const uint64_t t = t0 + j;
-                const uint32_t m = __shfl_sync(0xFFFFFFFFu, ml, j);
-                uint64_t o = P.key_off[t];
-                const uint64_t *rr = P.recs + t * P.unit_cap;
-                const uint64_t tile_start = t << P.unit_shift;
-                for (uint32_t i0 = 0; i0 < m; i0 += 32) {
-                    const uint32_t i = i0 + lane;
-                    uint64_t r = 0;
-                    uint32_t L = 0;
-                    if (i < m) {
-                        r = rr[i];
-                        L = fin_len_c(P, (uint32_t)r);
-                    }
-                    uint32_t inc = L;
+//
+// A warp takes `span` consecutive units (32, or 4 when there are few, so that
+// the chains of dependent loads run in more warps) and deals those that have
+// records out to groups of eight lanes, one record a lane: four units at a
+// time, each with one round trip for its records and one for its outputs.
+// Units with more records take the whole warp, 32 records at a time.  A
+// record's keys follow those of the records at lower positions: the earlier
+// lanes' where the records lie in position order, else (the window kernel's
+// units, at most 32 records) those found lower by comparing.
+constexpr uint32_t EXPAND_GROUP = 8;  // lanes, and most records, of a group's unit
+constexpr uint32_t EXPAND_SPAN = 32, EXPAND_SPAN_FEW = 4;
+
+// Keys before this lane's record among the `width` lanes of its group; width
+// is the unit's lanes (EXPAND_GROUP or 32).
+template <uint32_t WIDTH>
+__device__ __forceinline__ uint32_t keys_before(uint32_t pos, uint32_t L, bool unordered, uint32_t lane) {
+    if (unordered) {
+        uint32_t lower = 0;
 #pragma unroll
-                    for (int s = 1; s < 32; s <<= 1) {
-                        const uint32_t nb = __shfl_up_sync(0xFFFFFFFFu, inc, s);
-                        if (lane >= (uint32_t)s) inc += nb;
-                    }
-                    if (L) {
-                        const uint32_t *ids = fin_ids_c(P, (uint32_t)r);
-                        const uint64_t pk = (P.pos_base + tile_start + (r >> 32)) << PFAC_ID_BITS;
-                        uint64_t oo = o + inc - L;
-                        for (uint32_t e = 0; e < L; e++, oo++)
-                            if (oo < P.cap) P.out[oo] = pk | __ldg(ids + e);
-                    }
-                    o += __shfl_sync(0xFFFFFFFFu, inc, 31);
+        for (uint32_t x = 0; x < WIDTH; x++) {
+            const uint32_t px = __shfl_sync(0xFFFFFFFFu, pos, x, WIDTH);
+            const uint32_t lx = __shfl_sync(0xFFFFFFFFu, L, x, WIDTH);
+            if (px < pos) lower += lx;
+        }
+        return lower;
+    }
+    uint32_t inc = L;
+#pragma unroll
+    for (uint32_t s = 1; s < WIDTH; s <<= 1) {
+        const uint32_t nb = __shfl_up_sync(0xFFFFFFFFu, inc, s, WIDTH);
+        if ((lane & (WIDTH - 1)) >= s) inc += nb;
+    }
+    return inc - L;
+}
+
+__device__ __forceinline__ void write_keys(const MatchParams &P, uint64_t r, uint32_t L, uint64_t t,
+                                           uint64_t o) {
+    if (!L) return;
+    const uint32_t *ids = fin_ids_c(P, (uint32_t)r);
+    const uint64_t pk = (P.pos_base + (t << P.unit_shift) + (r >> 32)) << PFAC_ID_BITS;
+    for (uint32_t e = 0; e < L; e++, o++)
+        if (o < P.cap) P.out[o] = pk | __ldg(ids + e);
+}
+
+__global__ void __launch_bounds__(256) k_expand(const MatchParams P, const uint32_t span) {
+    __shared__ bool last;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t grp = lane / EXPAND_GROUP, gl = lane % EXPAND_GROUP;
+    const uint64_t gwarp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    const bool un = P.unordered != 0;
+    for (uint64_t t0 = gwarp * span; t0 < P.n_tiles; t0 += nwarps * span) {
+        const uint64_t tl = t0 + lane;
+        const bool mine = lane < span && tl < P.n_tiles;
+        const uint32_t ml = mine ? P.tile_m[tl] : 0u;
+        uint32_t few = __ballot_sync(0xFFFFFFFFu, ml != 0 && ml <= EXPAND_GROUP);
+        uint32_t many = __ballot_sync(0xFFFFFFFFu, ml > EXPAND_GROUP && ml <= P.unit_cap);
+        const uint64_t ol = ml != 0 && ml <= P.unit_cap ? P.key_off[tl] : 0ull;
+        while (few) {
+            // the group's unit: the grp-th set bit
+            uint32_t f = few;
+            for (uint32_t x = 0; x < grp; x++) f &= f - 1;
+            const uint32_t j = f ? __ffs(f) - 1 : 0u;
+            const uint32_t m = __shfl_sync(0xFFFFFFFFu, ml, j);
+            const uint64_t o = __shfl_sync(0xFFFFFFFFu, ol, j);
+            uint64_t r = 0;
+            uint32_t L = 0;
+            if (f && gl < m) {
+                r = P.recs[(t0 + j) * P.unit_cap + gl];
+                L = fin_len_c(P, (uint32_t)r);
+            }
+            const uint32_t before = keys_before<EXPAND_GROUP>((uint32_t)(r >> 32), L, un, lane);
+            write_keys(P, r, L, t0 + j, o + before);
+#pragma unroll
+            for (uint32_t x = 0; x < 32 / EXPAND_GROUP; x++) few &= few - 1;
+        }
+        while (many) {
+            const uint32_t j = __ffs(many) - 1;
+            many &= many - 1;
+            const uint64_t t = t0 + j;
+            const uint32_t m = __shfl_sync(0xFFFFFFFFu, ml, j);
+            uint64_t o = __shfl_sync(0xFFFFFFFFu, ol, j);
+            for (uint32_t i0 = 0; i0 < m; i0 += 32) {
+                const uint32_t i = i0 + lane;
+                uint64_t r = 0;
+                uint32_t L = 0;
+                if (i < m) {
+                    r = P.recs[t * P.unit_cap + i];
+                    L = fin_len_c(P, (uint32_t)r);
                 }
+                const uint32_t before = keys_before<32>((uint32_t)(r >> 32), L, un, lane);
+                write_keys(P, r, L, t, o + before);
+                // (unordered units end after one round)
+                o += __shfl_sync(0xFFFFFFFFu, before + L, 31);
             }
         }
     }
@@ -323,18 +372,31 @@ struct Plan {
     // its own (one bitmap copy, entries through L2)
     size_t smem_emit;
     uint32_t e_tbl_words, e_tbl_m_words;
+    // the window kernel takes the scan (the fields above then describe the
+    // plan that its options would otherwise run): the prefix bitmap its
+    // candidates are tested against, its words in shared memory
+    bool win;
+    uint32_t wf_k, wf_words;
+    size_t smem_win;
+    void *kernel_win, *kernel_win_small;
 };
 
 enum { SCAN_QUEUED = 1, SCAN_REGISTER = 2, SCAN_SERIAL = 3 };
 
 struct WsLayout {
     uint64_t hdr, tile_m, tile_k, key_off, chunk, ovf, recs, bounds, defer, dbatch, total;
-    uint32_t n_tiles, n_chunks, defer_cap, dbatch_cap;
+    uint64_t wbuf;
+    uint32_t n_tiles, n_chunks, defer_cap, dbatch_cap, wbuf_cap;
 };
 
 // entries per slice the resolver kernel's buffer holds (more go to the
 // scan kernel's own resolution)
 constexpr uint32_t DEFER_PER_UNIT = 8;
+// entries per slice of the window kernel's buffer (8 bytes each)
+constexpr uint32_t WBUF_PER_UNIT = 16;
+// pairs of slices per SM up to which the window kernel reads its filter
+// through L2
+constexpr uint32_t WIN_SMALL_PAIRS = 16;
 
 static inline uint64_t al256(uint64_t x) { return (x + 255) & ~255ull; }
 
@@ -362,11 +424,16 @@ static WsLayout ws_layout(uint64_t n_bytes, uint32_t n_seg, const Plan &pl) {
     L.bounds = put(n_seg > 1 ? (pl.queued ? nt * 4 : nt * SEGW * 4) : 0);
     // register-staged plans: the queues handed to the resolver kernel (at
     // most one batch per slice, plus each warp's last)
-    const uint64_t dcap = pl.defer ? std::min<uint64_t>(nt * DEFER_PER_UNIT, 0xFFFFFF00ull) : 0;
+    const bool defer = pl.defer && !pl.win;
+    const uint64_t dcap = defer ? std::min<uint64_t>(nt * DEFER_PER_UNIT, 0xFFFFFF00ull) : 0;
     L.defer_cap = (uint32_t)dcap;
-    L.dbatch_cap = pl.defer ? (uint32_t)std::min<uint64_t>(nt + 4096, 0xFFFFFF00ull) : 0u;
+    L.dbatch_cap = defer ? (uint32_t)std::min<uint64_t>(nt + 4096, 0xFFFFFF00ull) : 0u;
     L.defer = put(dcap * 16);
     L.dbatch = put((uint64_t)L.dbatch_cap * 8);
+    // the window kernel's entries (the counter runs at most one reservation
+    // per warp past the capacity)
+    L.wbuf_cap = pl.win ? (uint32_t)std::min<uint64_t>(nt * WBUF_PER_UNIT, 0xF0000000ull) : 0u;
+    L.wbuf = put((uint64_t)L.wbuf_cap * 8);
     L.total = o;
     return L;
 }
@@ -533,7 +600,7 @@ static int make_plan_r(const pfac_table *t, uint32_t k, int var, uint32_t masks,
     return PFAC_OK;
 }
 
-static int make_plan(const pfac_table *t, const pfac_match_opts *opts, Plan *pl) {
+static int make_scan_plan(const pfac_table *t, const pfac_match_opts *opts, Plan *pl) {
     const DevTable &T = t->dev;
     memset(pl, 0, sizeof(*pl));
     // the dense layout runs the compressed layout's kernels over its
@@ -816,6 +883,45 @@ static int make_plan(const pfac_table *t, const pfac_match_opts *opts, Plan *pl)
     return PFAC_OK;
 }
 
+// The plan of a call: the scan plan its options ask for and, when they leave
+// every choice to the library and the table has no tuned one, the window
+// kernel over the table's filter in place of that scan.  The emit pass, which
+// re-scans slices with more matches than their records, stays the plan's own.
+static int make_plan(const pfac_table *t, const pfac_match_opts *opts, Plan *pl) {
+    const int rc = make_scan_plan(t, opts, pl);
+    if (rc != PFAC_OK) return rc;
+    const DevTable &T = t->dev;
+    if (!T.H || T.dag || pl->kind == SCAN_SERIAL || pl->unit_cap != (uint32_t)SCAP) return PFAC_OK;
+    if (opts && (opts->variant || opts->prefix_depth || opts->ctas_per_sm || opts->bitmap_copies ||
+                 opts->child_masks || opts->gram_filter || opts->prefix_bytes ||
+                 opts->warps_per_cta || opts->scan_kernel || opts->test_wait_limit_us ||
+                 opts->test_withhold_slice || opts->records_per_slice || opts->resolver))
+        return PFAC_OK;
+    if (t->tuned_variant || t->tuned_k || t->tuned_nw || t->tuned_kernel) return PFAC_OK;
+    // shared memory: the filter's copies, the warps' queues, then the deepest
+    // prefix bitmap held that still fits (none: candidates are tested through L2)
+    const size_t fixed = ((size_t)T.w_words << T.w_rep) * 4 + WNW * WQCAP * 4;
+    if (fixed > SMEM_LIMIT) return PFAC_OK;
+    pl->wf_k = pl->k;
+    for (uint32_t k = t->kmin; k <= pl->k; k++) {
+        const uint64_t fw = ((1ull << (k * T.bps)) + 31) / 32;
+        if (fw % 4 == 0 && fixed + fw * 4 <= SMEM_LIMIT) {
+            pl->wf_k = k;
+            pl->wf_words = (uint32_t)fw;
+        }
+    }
+    pl->smem_win = fixed + (size_t)pl->wf_words * 4;
+    pl->kernel_win = scan_kernel_w(T, T.w_rep ? WT_COPIES : WT_ONE);
+    pl->kernel_win_small = scan_kernel_w(T, WT_L2);
+    pl->kernel_res = wresolve_kernel((int)T.W);
+    if (!pl->kernel_win || !pl->kernel_win_small || !pl->kernel_res) {
+        pl->kernel_res = pl->defer ? resolve_kernel((int)T.W) : nullptr;
+        return PFAC_OK;
+    }
+    pl->win = true;
+    return PFAC_OK;
+}
+
 static std::mutex g_attr_mu;
 
 static int prepare_kernel(void *fn, size_t smem) {
@@ -957,7 +1063,7 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
                          (unsigned long long)workspace_bytes, (unsigned long long)L.total);
     const bool reg = pl.kind == SCAN_REGISTER;
     const size_t smem_emit = reg ? pl.smem_emit : pl.smem;
-    rc = prepare_kernel(pl.kernel, pl.smem);
+    rc = pl.win ? prepare_kernel(pl.kernel_win, pl.smem_win) : prepare_kernel(pl.kernel, pl.smem);
     if (!rc && pl.kernel_emit != pl.kernel) rc = prepare_kernel(pl.kernel_emit, smem_emit);
     if (rc) return rc;
 
@@ -1013,7 +1119,21 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
     P.wait_limit_ns = opts && opts->test_wait_limit_us ? (uint64_t)opts->test_wait_limit_us * 1000
                                                        : WAIT_LIMIT_NS;
     P.withhold_unit = opts && opts->test_withhold_slice ? opts->test_withhold_slice - 1 : UNIT_NONE;
-    if (pl.defer) {
+    if (pl.win) {
+        const DevTable &T = t->dev;
+        const uint32_t bits = T.w_packed ? 2 * T.w_gw : 8 * T.w_gw;
+        P.wbuf = (uint64_t *)(W + L.wbuf);
+        P.wbuf_cap = L.wbuf_cap;
+        P.w_words = T.w_words;
+        P.w_rep = T.w_rep;
+        P.w_gm = gram_mul(bits);
+        P.w_glen = T.w_glen;
+        P.w_badmask = T.w_short ? 0x01010101u * ((0xFFu << T.bps) & 0xFFu) : 0u;
+        P.wf = T.F[pl.wf_k];
+        P.wf_words = pl.wf_words;
+        P.wf_k = pl.wf_k;
+        P.unordered = 1;
+    } else if (pl.defer) {
         P.defer = (uint4 *)(W + L.defer);
         P.defer_cap = L.defer_cap;
         P.dbatch = (uint2 *)(W + L.dbatch);
@@ -1039,13 +1159,23 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
     const uint32_t grid = (uint64_t)nsm * cps < want ? (uint32_t)nsm * cps : (uint32_t)want;
     if (e == cudaSuccess && opts && opts->ev_scan_begin)
         e = cudaEventRecord((cudaEvent_t)opts->ev_scan_begin, st);
-    if (e == cudaSuccess && P.n_tiles) {
+    if (e == cudaSuccess && P.n_tiles && pl.win) {
+        // few pairs of slices: one warp each, the filter read through L2
+        const uint32_t n_pairs = (P.n_tiles + 1) / 2;
+        const bool small = n_pairs <= (uint32_t)nsm * WIN_SMALL_PAIRS;
+        const uint32_t nw = small ? WNW_SMALL : WNW;
+        const uint32_t need = (n_pairs + nw - 1) / nw;
+        void *args[] = {&P};
+        e = cudaLaunchKernel(small ? pl.kernel_win_small : pl.kernel_win,
+                             dim3(small || need < (uint32_t)nsm ? need : (uint32_t)nsm), dim3(nw * 32),
+                             args, small ? (size_t)WNW_SMALL * WQCAP * 4 : pl.smem_win, st);
+    } else if (e == cudaSuccess && P.n_tiles) {
         int emit = 0;
         void *args[] = {&P, &emit};
         e = cudaLaunchKernel(pl.kernel, dim3(grid), dim3(nthreads), args, pl.smem, st);
     }
-    if (e == cudaSuccess && P.n_tiles && pl.defer) {
-        // the handed-over queues: prefix bitmap, counts and entries through
+    if (e == cudaSuccess && P.n_tiles && (pl.win || pl.defer)) {
+        // the handed-over queues (or the window kernel's entries): prefix bitmap, counts and entries through
         // L2 (one bitmap copy)
         MatchParams P3 = P;
         P3.rep_log2 = 0;
@@ -1093,11 +1223,11 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
     if (e == cudaSuccess && opts && opts->ev_emit_end)
         e = cudaEventRecord((cudaEvent_t)opts->ev_emit_end, st);
     if (e == cudaSuccess) {
-        const uint64_t units = P.n_tiles ? P.n_tiles : 1;
-        uint64_t blocks = (units + 255) / 256;
         const uint64_t maxb = (uint64_t)nsm * 8;
+        const uint32_t span = (uint64_t)P.n_tiles <= maxb * 8 * EXPAND_SPAN_FEW ? EXPAND_SPAN_FEW : EXPAND_SPAN;
+        uint64_t blocks = ((uint64_t)P.n_tiles + 8 * span - 1) / (8 * span);
         if (blocks > maxb) blocks = maxb;
-        k_expand<<<(uint32_t)blocks, 256, 0, st>>>(P);
+        k_expand<<<(uint32_t)(blocks ? blocks : 1), 256, 0, st>>>(P, span);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess)

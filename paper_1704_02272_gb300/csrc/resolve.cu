@@ -1,5 +1,5 @@
-// Instances of the resolver kernel, one per record format.
-#include "kernels_r.cuh"
+// Instances of the resolver kernels, one per record format.
+#include "kernels_w.cuh"
 
 namespace pfac {
 
@@ -10,6 +10,17 @@ void *resolve_kernel(int w) {
         case 2: return (void *)k_resolve<2>;
         case 3: return (void *)k_resolve<3>;
         case 8: return (void *)k_resolve<8>;
+        default: return nullptr;
+    }
+}
+
+void *wresolve_kernel(int w) {
+    switch (w) {
+        case 0: return (void *)k_wresolve<0>;
+        case 1: return (void *)k_wresolve<1>;
+        case 2: return (void *)k_wresolve<2>;
+        case 3: return (void *)k_wresolve<3>;
+        case 8: return (void *)k_wresolve<8>;
         default: return nullptr;
     }
 }

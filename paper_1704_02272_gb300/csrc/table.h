@@ -139,6 +139,20 @@ __host__ __device__ inline uint32_t child_hash(uint32_t c, uint32_t sigma) {
     return sigma <= 32 ? c : ((c ^ (c >> 5)) & 31u);
 }
 
+// Window filter (the window kernel's table): words of 32 bits over strings of
+// g symbols.  A string's word is the top of its hash y scaled to w_words,
+// y = t * win_mul(gw) (+ t1 * WIN_MUL2 with five raw symbols), t the window's
+// first 32 bits (raw bytes, first symbol lowest, or 2-bit symbols), t1 those
+// one symbol on; gw is the symbols hashed.  Its NB bits within the word are
+// the low 5 bits of the window at fixed symbol offsets: 2, 0, 1 with raw
+// bytes, 0, 3, 6 with 2-bit symbols.  H holds every g-string that stands at
+// an offset 0 .. S - 1 of an occurrence of a pattern, patterns that end
+// inside it with every completion over the packed symbol values.
+constexpr uint32_t WIN_MUL2 = 0x85EBCA6Bu;  // an odd constant with mixed bits (MurmurHash3's finaliser)
+__host__ __device__ inline uint32_t win_off(uint32_t packed, uint32_t i) {
+    return packed ? 3 * i : (i == 0 ? 2u : i - 1u);
+}
+
 struct DevTable {
     uint32_t sigma;
     uint32_t W;           // record format: 0 (packed), 1, 2 or 8 (bitmap words)
@@ -186,6 +200,16 @@ struct DevTable {
     uint32_t side_slots;      // slots of the side table
     const uint64_t *side_keys;
     const uint32_t *side_vals;
+    // window filter (nullptr when the pattern set makes none that pays)
+    const uint32_t *H;
+    uint32_t w_words;         // words of H (a multiple of 32)
+    uint32_t w_rep;           // copies in shared memory (log2)
+    uint32_t w_stride;        // S: 1, 2, 4, 8 or 16
+    uint32_t w_nb;            // bits tested per window
+    uint32_t w_gw;            // symbols hashed
+    uint32_t w_glen;          // symbols a window's test reads
+    uint32_t w_packed;        // 1: windows of 2-bit symbols; 0: of raw bytes
+    uint32_t w_short;         // 1: some patterns end inside a window (completions in H)
 };
 
 }  // namespace pfac

@@ -6,6 +6,7 @@
 // offset into the blob, NO_SECTION for none; the table statistics, the
 // prefix depths held, the tuned defaults), then the blob bytes.
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdio.h>
 #include <string.h>
 #include <unistd.h>
@@ -48,6 +49,12 @@ struct FileMeta {
     double match_density;
 };
 
+// Files written before the window filter existed hold a DevTable that ends
+// where its fields begin; they load as tables without one.
+constexpr size_t DEV_OLD = offsetof(DevTable, H);
+constexpr size_t META_OLD = sizeof(FileMeta) - (sizeof(DevTable) - DEV_OLD);
+static_assert(offsetof(FileMeta, info) == sizeof(DevTable), "description follows the table");
+
 // Calls fn(p) with a reference to every pointer field p of a DevTable.
 template <class Fn>
 void for_each_section(DevTable &d, Fn &&fn) {
@@ -72,6 +79,7 @@ void for_each_section(DevTable &d, Fn &&fn) {
     fn(d.ind);
     fn(d.side_keys);
     fn(d.side_vals);
+    fn(d.H);
 }
 
 template <class T>
@@ -100,9 +108,9 @@ struct Fnv64 {
     }
 };
 
-uint64_t checksum(const FileMeta &m, const uint8_t *blob, uint64_t n) {
+uint64_t checksum(const void *meta, uint64_t meta_bytes, const uint8_t *blob, uint64_t n) {
     Fnv64 f;
-    f.add(&m, sizeof m);
+    f.add(meta, meta_bytes);
     f.add(blob, n);
     return f.h;
 }
@@ -177,6 +185,18 @@ int check_meta(FileMeta &m, const uint8_t *blob, uint64_t blob_bytes) {
     span(d.ind, d.ind_words, true);
     span(d.side_keys, d.dag ? (uint64_t)d.side_slots : 0, d.dag != 0);
     span(d.side_vals, d.dag ? (uint64_t)d.side_slots : 0, d.dag != 0);
+    if ((uint64_t)(uintptr_t)d.H != NO_SECTION) {
+        // window filter: the kernels' strides and bit counts, words in whole
+        // vectors, and room in shared memory
+        const uint32_t S = d.w_stride;
+        if (!(S == 1 || S == 2 || S == 4 || S == 8 || S == 16) || d.w_nb < 1 || d.w_nb > 3 ||
+            d.w_rep > 5 || d.w_words < 32 || d.w_words % 32 || ((uint64_t)d.w_words << d.w_rep) > 49152 ||
+            d.w_packed > 1 || d.w_packed != (d.bps == 2 ? 1u : 0u) || d.bps < 2 || d.w_gw < 1 ||
+            d.w_glen > (d.w_packed ? 16u : 5u) || d.w_glen < d.w_gw)
+            return bad("window filter");
+        span(d.H, d.w_words, true);
+        if ((uint64_t)(uintptr_t)d.H % 16) return bad("section offset");
+    }
     if (rc != PFAC_OK) return rc;
     // truncated tables: pattern j is pat[pat_off[j] .. pat_off[j + 1])
     const uint64_t o_po = (uint64_t)(uintptr_t)d.pat_off, o_pb = (uint64_t)(uintptr_t)d.pat;
@@ -247,7 +267,7 @@ extern "C" int pfac_table_save(const pfac_table *t, const char *path) {
         h.info_bytes = sizeof(pfac_table_info_t);
         h.meta_bytes = sizeof(FileMeta);
         h.blob_bytes = t->blob_bytes;
-        h.checksum = checksum(m, blob, t->blob_bytes);
+        h.checksum = checksum(&m, sizeof m, blob, t->blob_bytes);
 
         const std::string dst(path);
         const std::string tmp = dst + ".tmp." + std::to_string((long)getpid());
@@ -283,6 +303,7 @@ extern "C" int pfac_table_load(const char *path, uint32_t flags, void *cuda_stre
         if (!f) return io_error("pfac_table_load", "cannot open", src);
         FileHeader h;
         FileMeta m;
+        std::vector<uint8_t> meta;  // as the file holds it
         std::vector<uint8_t> blob;
         int rc = PFAC_OK;
         long long fsize = -1;
@@ -293,24 +314,29 @@ extern "C" int pfac_table_load(const char *path, uint32_t flags, void *cuda_stre
             rc = set_error(PFAC_EFORMAT, "pfac_table_load: %s is shorter than a header", path);
         } else if (memcmp(h.magic, MAGIC, sizeof MAGIC) != 0 || h.endian != ENDIAN_MARK) {
             rc = set_error(PFAC_EFORMAT, "pfac_table_load: %s is not a table file", path);
-        } else if (h.version != FORMAT_VERSION || h.devtable_bytes != sizeof(DevTable) ||
-                   h.info_bytes != sizeof(pfac_table_info_t) || h.meta_bytes != sizeof(FileMeta)) {
+        } else if (h.version != FORMAT_VERSION || h.info_bytes != sizeof(pfac_table_info_t) ||
+                   !((h.devtable_bytes == sizeof(DevTable) && h.meta_bytes == sizeof(FileMeta)) ||
+                     (h.devtable_bytes == DEV_OLD && h.meta_bytes == META_OLD))) {
             rc = set_error(PFAC_EFORMAT,
                            "pfac_table_load: %s was written by another format version (%u; this "
                            "library reads %u)", path, h.version, FORMAT_VERSION);
-        } else if ((uint64_t)fsize != sizeof h + sizeof m + h.blob_bytes) {
+        } else if ((uint64_t)fsize != sizeof h + (uint64_t)h.meta_bytes + h.blob_bytes) {
             rc = set_error(PFAC_EFORMAT, "pfac_table_load: %s has %lld bytes, its header says %llu",
-                           path, fsize, (unsigned long long)(sizeof h + sizeof m + h.blob_bytes));
-        } else if (fread(&m, sizeof m, 1, f) != 1) {
+                           path, fsize, (unsigned long long)(sizeof h + (uint64_t)h.meta_bytes + h.blob_bytes));
+        } else if (meta.resize(h.meta_bytes), fread(meta.data(), h.meta_bytes, 1, f) != 1) {
             rc = io_error("pfac_table_load", "cannot read", src);
         } else {
+            memset(&m, 0, sizeof m);
+            memcpy(&m.dev, meta.data(), h.devtable_bytes);
+            memcpy(&m.info, meta.data() + h.devtable_bytes, h.meta_bytes - h.devtable_bytes);
+            if (h.devtable_bytes == DEV_OLD) m.dev.H = (const uint32_t *)(uintptr_t)NO_SECTION;
             blob.resize(h.blob_bytes);
             if (h.blob_bytes && fread(blob.data(), h.blob_bytes, 1, f) != 1)
                 rc = io_error("pfac_table_load", "cannot read", src);
         }
         fclose(f);
         if (rc != PFAC_OK) return rc;
-        if (checksum(m, blob.data(), h.blob_bytes) != h.checksum)
+        if (checksum(meta.data(), meta.size(), blob.data(), h.blob_bytes) != h.checksum)
             return set_error(PFAC_EFORMAT, "pfac_table_load: %s: checksum mismatch", path);
         rc = check_meta(m, blob.data(), h.blob_bytes);
         if (rc != PFAC_OK) return rc;
