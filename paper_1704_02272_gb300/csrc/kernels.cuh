@@ -10,10 +10,11 @@
 // its slot; the tile's (position, fin) records go to a per-tile region of the
 // workspace and the tile's match and key counts to per-unit counters.
 //
-// Ordering kernels (match.cu): k_reduce scans the per-unit key counts,
-// k_offsets turns them into per-unit output offsets, k_expand writes the
-// sorted keys of each unit from its records, and units whose records did not
-// fit re-run the scan kernel in emit mode, which writes keys directly.  No
+// Ordering kernels (match.cu): k_reduce sums the key counts of chunks of
+// units, k_expand turns them into output offsets and writes the sorted keys of
+// each unit from its records, and units whose records did not fit re-run the
+// scan kernel in emit mode, which writes keys directly and publishes the
+// call's status.  No
 // kernel waits on another CTA; the only waits are mbarrier waits, each bounded
 // by a wall-clock limit after which the kernel records PFAC_ETIMEOUT.
 #pragma once
@@ -55,8 +56,8 @@ constexpr int VAR_RES = 16;
 struct WsHeader {
     int32_t status;
     uint32_t ovf_count;
-    uint32_t done_reduce;
-    uint32_t done_expand;
+    uint32_t done_emit;      // CTAs of the emit pass that have finished
+    uint32_t pad0;
     uint32_t defer_entries;  // queue entries handed to the resolver kernel
     uint32_t defer_batches;  // and their batches
     uint32_t pad[10];
@@ -78,10 +79,11 @@ struct MatchParams {
     // workspace
     WsHeader *hdr;
     uint32_t *tile_m;     // per unit: records kept, or more than unit_cap
-    uint64_t *tile_k;     // per unit: keys
-    uint64_t *key_off;    // per unit: first output slot
-    uint64_t *chunk;      // n_chunks sums, then n_chunks offsets
-    uint32_t n_chunks;
+    uint64_t *tile_k;     // per unit: keys (unordered: and records, above UNIT_KEY_BITS)
+    uint64_t *key_off;    // per unit of the emit pass: first output slot
+    uint64_t *chunk;      // keys per chunk of 2^chunk_shift units
+    uint32_t chunk_shift;
+    uint32_t chunk_adds;  // matches add to their chunk's count as they are found
     uint32_t *ovf_list;
     uint64_t *recs;
     uint32_t *tile_bounds;  // tile-synchronous kernel: segment ends per tile
@@ -132,6 +134,8 @@ struct MatchParams {
 };
 
 constexpr uint32_t UNIT_NONE = 0xFFFFFFFFu;
+// a unit's keys fit: 512 positions of at most 2^24 ids each
+constexpr int UNIT_KEY_BITS = 40;
 
 // The bounds-checked build (compiled with PFAC_CHECKED, a separate library):
 // the compressed-layout kernels pass every table, shared-memory, queue and
@@ -235,6 +239,24 @@ __device__ __forceinline__ bool cons_bar_and(bool v) {
         : "r"((uint32_t)v), "n"(NCONS)
         : "memory");
     return r != 0;
+}
+
+// ------------------------------------------------------------ status -------
+
+__device__ __forceinline__ int32_t status_code(int32_t st) {
+    if (st & ST_BADSEG) return PFAC_EINVAL;
+    if (st & ST_TIMEOUT) return PFAC_ETIMEOUT;
+    if (st & ST_DEVICE) return PFAC_EDEVICE;
+    return PFAC_OK;
+}
+
+// Called once per CTA by one thread, after the CTA's work: the last of `ctas`
+// callers publishes the call's status.
+__device__ __forceinline__ void publish_status(const MatchParams &P, uint32_t ctas) {
+    __threadfence();
+    if (atomicAdd(&P.hdr->done_emit, 1u) != ctas - 1) return;
+    __threadfence();
+    if (P.d_status) *P.d_status = status_code(*(volatile int32_t *)&P.hdr->status);
 }
 
 // ------------------------------------------------------------ outputs ------
@@ -455,7 +477,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_scan_dense(const MatchParams P,
 
     const uint32_t tid = threadIdx.x;
     const uint32_t n_work = emit ? *(volatile uint32_t *)&P.hdr->ovf_count : P.n_tiles;
-    if (blockIdx.x >= n_work) return;
+    if (blockIdx.x >= n_work) {
+        if (emit && n_work == 0 && blockIdx.x == 0 && tid == 0) publish_status(P, 1);
+        return;
+    }
 
     if (tid == 0) {
         for (int s = 0; s < STAGES; s++) {
@@ -582,6 +607,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_scan_dense(const MatchParams P,
                     if (o < P.cap) P.out[o] = pk | __ldg(ids + e);
             }
         }
+    }
+    if (emit) {
+        cons_bar();
+        if (tid == 0) publish_status(P, gridDim.x < n_work ? gridDim.x : n_work);
     }
 }
 

@@ -140,15 +140,21 @@ __device__ __forceinline__ uint32_t w_filter(const uint32_t (&w)[9], const WCons
 }
 
 // One match: a record in the slice's space while it has room (in any order),
-// the slice's key count; the first match past the space lists the slice for
-// the emit pass.
+// and the slice's counts: records above bit UNIT_KEY_BITS of its word, keys
+// below, so that one atomic takes the slot and counts the keys.  The first
+// match past the space lists the slice for the emit pass.  With few slices
+// the chunks' key counts are added up here too; with many, neighbouring
+// matches would queue on one chunk's word (1 GiB of packets: 0.8 instead of
+// 0.36 ms), and k_reduce sums them.
 __device__ __forceinline__ void w_emit(const MatchParams &P, uint32_t u, uint32_t pos, uint32_t fin) {
     u = (uint32_t)chk(P, u, P.n_tiles);
     const uint32_t cap = P.unit_cap;
-    const uint32_t rank = atomicAdd(P.tile_m + u, 1u);
+    const unsigned long long keys = fin_len_c(P, fin);
+    const uint32_t rank = (uint32_t)(atomicAdd((unsigned long long *)(P.tile_k + u),
+                                               (1ull << UNIT_KEY_BITS) | keys) >> UNIT_KEY_BITS);
     if (rank < cap) P.recs[(size_t)u * cap + rank] = ((uint64_t)pos << 32) | fin;
     else if (rank == cap) P.ovf_list[chk(P, atomicAdd(&P.hdr->ovf_count, 1u), P.n_tiles)] = u;
-    atomicAdd((unsigned long long *)(P.tile_k + u), (unsigned long long)fin_len_c(P, fin));
+    if (P.chunk_adds) atomicAdd((unsigned long long *)(P.chunk + (u >> P.chunk_shift)), keys);
 }
 
 // Walk limit of start p of slice u, relative to the slice start: the first
@@ -159,7 +165,10 @@ __device__ __forceinline__ uint32_t w_limit(const MatchParams &P, uint32_t u, ui
     const uint64_t remain = P.n - ustart;
     const uint32_t rem = remain < LIM_MAX ? (uint32_t)remain : LIM_MAX;
     if (P.n_seg <= 1) return rem;
+    // (bounded: offsets out of order leave some indices unwritten)
     uint32_t lo = __ldg(P.unit_seg + u), hi = u + 1 < P.n_tiles ? __ldg(P.unit_seg + u + 1) : P.n_seg;
+    lo = lo < P.n_seg ? lo : P.n_seg;
+    hi = hi < P.n_seg ? hi : P.n_seg;
     while (lo < hi) {
         const uint32_t mid = (lo + hi) >> 1;
         if (__ldg(P.seg + mid) > p) hi = mid; else lo = mid + 1;
@@ -369,6 +378,8 @@ __global__ void __launch_bounds__((TB == WT_L2 ? WNW_SMALL : WNW) * 32, 1)
     const uint32_t n_pairs = (P.n_tiles + 1) >> 1;
     const uint32_t gw = blockIdx.x * NW + warp, gstride = gridDim.x * NW;
     if (blockIdx.x * NW >= n_pairs) return;
+
+    if (P.n_seg > 1) unit_segments(P, gw, gstride, lane);
 
     // shared memory: H (all copies), the prefix bitmap, the queues
     const uint32_t hwords = TB == WT_L2 ? 0u : P.w_words << P.w_rep;

@@ -73,8 +73,15 @@ static void *scan_kernel_w(const DevTable &T, int tb) {
     }
 }
 
-constexpr int CHUNK = 1024;      // tiles per chunk of the key-count scan
-constexpr int RT = 1024;         // threads of the scan/offset kernels
+// chunks of the key-count scan: the fewest units each (a power of two, 32 at
+// least) that keep their number within this
+constexpr uint32_t CHUNKS_MAX = 2048;
+constexpr uint32_t CHUNK_SHIFT_MIN = 5;
+static uint32_t chunk_shift(uint64_t n_units) {
+    uint32_t s = CHUNK_SHIFT_MIN;
+    while (((n_units + (1ull << s) - 1) >> s) > CHUNKS_MAX) s++;
+    return s;
+}
 
 // ------------------------------------------------ segment bounds per tile --
 
@@ -113,25 +120,10 @@ __global__ void k_bounds(const MatchParams P) {
     }
 }
 
-// Validates the offsets and records, per 512-byte unit of the queued scan
-// kernel, the index of the first offset beyond the unit start.
+// The segment data of the slice kernels (the window kernel does this itself).
 __global__ void k_unitseg(const MatchParams P) {
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    const uint64_t gt = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const uint64_t *seg = P.seg;
-    for (uint64_t s = gt; s < P.n_seg; s += stride)
-        if (__ldg(seg + s + 1) < __ldg(seg + s)) atomicOr(&P.hdr->status, ST_BADSEG);
-    if (gt == 0 && (__ldg(seg) != 0 || __ldg(seg + P.n_seg) != P.n))
-        atomicOr(&P.hdr->status, ST_BADSEG);
-    for (uint64_t u = gt; u < P.n_tiles; u += stride) {
-        const uint64_t start = u << P.unit_shift;
-        uint32_t lo = 1, hi = P.n_seg;
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (__ldg(seg + mid) > start) hi = mid; else lo = mid + 1;
-        }
-        P.unit_seg[u] = lo;
-    }
+    const uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x;
+    unit_segments(P, gt >> 5, (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
 }
 
 // ------------------------------------------------ key-count scan ----------
@@ -164,93 +156,33 @@ __device__ __forceinline__ uint64_t block_excl_scan(uint64_t v, uint64_t *sh, ui
     return r;
 }
 
-__device__ __forceinline__ int32_t status_code(int32_t st) {
-    if (st & ST_BADSEG) return PFAC_EINVAL;
-    if (st & ST_TIMEOUT) return PFAC_ETIMEOUT;
-    if (st & ST_DEVICE) return PFAC_EDEVICE;
-    return PFAC_OK;
-}
-
-// Chunk sums of the per-tile key counts; the last CTA scans the chunk sums,
-// writes the total match count and checks single-segment offsets.
-__global__ void __launch_bounds__(RT) k_reduce(const MatchParams P) {
+// Key counts of the chunks of units, where they are not added up as matches
+// are found.
+__global__ void __launch_bounds__(256) k_reduce(const MatchParams P) {
     __shared__ uint64_t sh[33];
-    __shared__ bool last;
-    const uint32_t c = blockIdx.x;
+    const uint64_t t0 = (uint64_t)blockIdx.x << P.chunk_shift;
     uint64_t sum = 0;
-    if (c < P.n_chunks) {
-        const uint64_t t0 = (uint64_t)c * CHUNK;
-        for (uint32_t i = threadIdx.x; i < CHUNK; i += RT) {
-            const uint64_t t = t0 + i;
-            if (t < P.n_tiles) sum += P.tile_k[t];
-        }
-    }
+    for (uint64_t i = threadIdx.x; i < (1ull << P.chunk_shift); i += 256)
+        if (t0 + i < P.n_tiles) sum += P.tile_k[t0 + i] & ((1ull << UNIT_KEY_BITS) - 1);
     uint64_t total;
     block_excl_scan(sum, sh, total);
-    if (threadIdx.x == 0) {
-        if (c < P.n_chunks) P.chunk[c] = total;
-        __threadfence();
-        last = atomicAdd(&P.hdr->done_reduce, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    uint64_t carry = 0;
-    for (uint32_t base = 0; base < P.n_chunks; base += RT) {
-        const uint32_t i = base + threadIdx.x;
-        const uint64_t v = i < P.n_chunks ? __ldcg(P.chunk + i) : 0;
-        uint64_t tot;
-        const uint64_t ex = block_excl_scan(v, sh, tot);
-        if (i < P.n_chunks) P.chunk[P.n_chunks + i] = carry + ex;
-        carry += tot;
-    }
-    if (threadIdx.x == 0) {
-        *P.d_count = carry;
-        if (P.n_seg <= 1) {
-            const bool ok = P.n_seg == 1 ? (P.seg[0] == 0 && P.seg[1] == P.n)
-                                         : (P.n == 0 && P.seg[0] == 0);
-            if (!ok) atomicOr(&P.hdr->status, ST_BADSEG);
-        }
-    }
+    if (threadIdx.x == 0) P.chunk[blockIdx.x] = total;
 }
 
-// Per-tile output offsets: chunk offset plus the scan inside the chunk.
-__global__ void __launch_bounds__(RT) k_offsets(const MatchParams P) {
-    __shared__ uint64_t sh[33];
-    const uint32_t c = blockIdx.x;
-    const uint64_t t0 = (uint64_t)c * CHUNK;
-    constexpr int PER = CHUNK / RT;
-    uint64_t v[PER];
-    uint64_t s = 0;
-#pragma unroll
-    for (int i = 0; i < PER; i++) {
-        const uint64_t t = t0 + threadIdx.x * PER + i;
-        v[i] = t < P.n_tiles ? P.tile_k[t] : 0;
-        s += v[i];
-    }
-    uint64_t total;
-    uint64_t ex = block_excl_scan(s, sh, total) + __ldcg(P.chunk + P.n_chunks + c);
-#pragma unroll
-    for (int i = 0; i < PER; i++) {
-        const uint64_t t = t0 + threadIdx.x * PER + i;
-        if (t < P.n_tiles) P.key_off[t] = ex;
-        ex += v[i];
-    }
-}
-
-// Writes the keys of every unit whose records were kept; the last CTA
-// publishes the call's status.
+// Output offsets and keys of one chunk of units per CTA; the last chunk's CTA
+// writes the total count.  A CTA adds up the counts of the chunks before its
+// own (at most CHUNKS_MAX) and scans its units' counts 8 * span at a time:
+// `span` consecutive units per warp, 32, or 4 when there are few, so that the
+// chains of dependent loads run in more warps.  Units whose records were not
+// kept get their offset stored for the emit pass.
 //
-// A warp takes `span` consecutive units (32, or 4 when there are few, so that
-// the chains of dependent loads run in more warps) and deals those that have
-// records out to groups of eight lanes, one record a lane: four units at a
+// A warp deals its units that have records out to groups of eight lanes, one record a lane: four units at a
 // time, each with one round trip for its records and one for its outputs.
 // Units with more records take the whole warp, 32 records at a time.  A
 // record's keys follow those of the records at lower positions: the earlier
 // lanes' where the records lie in position order, else (the window kernel's
 // units, at most 32 records) those found lower by comparing.
 constexpr uint32_t EXPAND_GROUP = 8;  // lanes, and most records, of a group's unit
-constexpr uint32_t EXPAND_SPAN = 32, EXPAND_SPAN_FEW = 4;
 
 // Keys before this lane's record among the `width` lanes of its group; width
 // is the unit's lanes (EXPAND_GROUP or 32).
@@ -285,19 +217,30 @@ __device__ __forceinline__ void write_keys(const MatchParams &P, uint64_t r, uin
 }
 
 __global__ void __launch_bounds__(256) k_expand(const MatchParams P, const uint32_t span) {
-    __shared__ bool last;
-    const uint32_t lane = threadIdx.x & 31;
+    __shared__ uint64_t sh[33];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t grp = lane / EXPAND_GROUP, gl = lane % EXPAND_GROUP;
-    const uint64_t gwarp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const bool un = P.unordered != 0;
-    for (uint64_t t0 = gwarp * span; t0 < P.n_tiles; t0 += nwarps * span) {
-        const uint64_t tl = t0 + lane;
-        const bool mine = lane < span && tl < P.n_tiles;
-        const uint32_t ml = mine ? P.tile_m[tl] : 0u;
+    const uint32_t c = blockIdx.x;
+    uint64_t base = 0;
+    {
+        uint64_t v = 0;
+        for (uint32_t i = threadIdx.x; i < c; i += 256) v += __ldcg(P.chunk + i);
+        block_excl_scan(v, sh, base);
+    }
+    const uint64_t c_end = ((uint64_t)c + 1) << P.chunk_shift;
+    const uint64_t t_end = c_end < P.n_tiles ? c_end : P.n_tiles;
+    for (uint64_t b0 = (uint64_t)c << P.chunk_shift; b0 < t_end; b0 += 8 * span) {
+        const uint64_t t0 = b0 + warp * span, tl = t0 + lane;
+        const bool mine = lane < span && tl < t_end;
+        const uint64_t kl = mine ? P.tile_k[tl] : 0ull;
+        const uint32_t ml = un ? (uint32_t)(kl >> UNIT_KEY_BITS) : (mine ? P.tile_m[tl] : 0u);
+        uint64_t tot;
+        const uint64_t ol = block_excl_scan(kl & ((1ull << UNIT_KEY_BITS) - 1), sh, tot) + base;
+        base += tot;
+        if (ml > P.unit_cap) P.key_off[tl] = ol;
         uint32_t few = __ballot_sync(0xFFFFFFFFu, ml != 0 && ml <= EXPAND_GROUP);
         uint32_t many = __ballot_sync(0xFFFFFFFFu, ml > EXPAND_GROUP && ml <= P.unit_cap);
-        const uint64_t ol = ml != 0 && ml <= P.unit_cap ? P.key_off[tl] : 0ull;
         while (few) {
             // the group's unit: the grp-th set bit
             uint32_t f = few;
@@ -337,15 +280,15 @@ __global__ void __launch_bounds__(256) k_expand(const MatchParams P, const uint3
             }
         }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(&P.hdr->done_expand, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (last && threadIdx.x == 0 && P.d_status) {
-        __threadfence();
-        *P.d_status = status_code(*(volatile int32_t *)&P.hdr->status);
+    if (threadIdx.x == 0 && c == gridDim.x - 1) {
+        *P.d_count = base;
+        if (P.n_seg <= 1) {
+            const bool ok = P.n_seg == 1 ? (P.seg[0] == 0 && P.seg[1] == P.n)
+                                         : (P.n == 0 && P.seg[0] == 0);
+            if (!ok) atomicOr(&P.hdr->status, ST_BADSEG);
+        }
+        // no unit, no emit pass: the status is published here
+        if (P.n_tiles == 0) publish_status(P, 1);
     }
 }
 
@@ -405,7 +348,8 @@ static WsLayout ws_layout(uint64_t n_bytes, uint32_t n_seg, const Plan &pl) {
     const uint64_t ub = 1ull << pl.unit_shift;
     const uint64_t nt = (n_bytes + ub - 1) / ub;
     L.n_tiles = (uint32_t)nt;
-    L.n_chunks = (uint32_t)((nt + CHUNK - 1) / CHUNK);
+    const uint32_t cs = chunk_shift(nt);
+    L.n_chunks = (uint32_t)((nt + (1ull << cs) - 1) >> cs);
     uint64_t o = 0;
     auto put = [&](uint64_t sz) {
         const uint64_t at = o;
@@ -413,10 +357,12 @@ static WsLayout ws_layout(uint64_t n_bytes, uint32_t n_seg, const Plan &pl) {
         return at;
     };
     L.hdr = put(sizeof(WsHeader));
-    L.tile_m = put(nt * 4);
+    // one memset zeroes the header and the counts (the record counts only
+    // where they are kept apart from the key counts)
+    L.chunk = put((uint64_t)CHUNKS_MAX * 8);
     L.tile_k = put(nt * 8);
+    L.tile_m = put(nt * 4);
     L.key_off = put(nt * 8);
-    L.chunk = put((uint64_t)L.n_chunks * 16);
     L.ovf = put(nt * 4);
     L.recs = put(nt * pl.unit_cap * 8);
     // segment data: per-tile lists (tile-synchronous kernel) or the first
@@ -1090,7 +1036,8 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
     P.tile_k = (uint64_t *)(W + L.tile_k);
     P.key_off = (uint64_t *)(W + L.key_off);
     P.chunk = (uint64_t *)(W + L.chunk);
-    P.n_chunks = (uint32_t)((P.n_tiles + CHUNK - 1) / CHUNK);
+    P.chunk_shift = chunk_shift(P.n_tiles);
+    const uint32_t n_chunks = (uint32_t)(((uint64_t)P.n_tiles + (1ull << P.chunk_shift) - 1) >> P.chunk_shift);
     P.ovf_list = (uint32_t *)(W + L.ovf);
     P.recs = (uint64_t *)(W + L.recs);
     P.tile_bounds = (uint32_t *)(W + L.bounds);
@@ -1133,6 +1080,7 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
         P.wf_words = pl.wf_words;
         P.wf_k = pl.wf_k;
         P.unordered = 1;
+        P.chunk_adds = P.chunk_shift == CHUNK_SHIFT_MIN;
     } else if (pl.defer) {
         P.defer = (uint4 *)(W + L.defer);
         P.defer_cap = L.defer_cap;
@@ -1144,12 +1092,13 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
     // take two slices each
     const uint32_t units_per_cta = pl.queued ? (reg ? 2 * pl.nw : pl.nw) : 1;
 
-    // header, and for the queued kernel the per-unit record and key counts
+    // header, and for the slice kernels the per-unit record and key counts
     // (the scan pass writes them only for units with kept survivors)
-    cudaError_t e = cudaMemsetAsync(P.hdr, 0, pl.queued ? L.key_off : sizeof(WsHeader), st);
+    cudaError_t e = cudaMemsetAsync(P.hdr, 0,
+                                    pl.win ? L.tile_m : (pl.queued ? L.key_off : sizeof(WsHeader)), st);
     const int nsm = sm_count();
     const uint32_t cps = opts && opts->ctas_per_sm ? opts->ctas_per_sm : 1;
-    if (e == cudaSuccess && n_segments > 1 && P.n_tiles) {
+    if (e == cudaSuccess && n_segments > 1 && P.n_tiles && !pl.win) {
         if (pl.queued) k_unitseg<<<nsm * 4, 256, 0, st>>>(P);
         else k_bounds<<<nsm * 2, 256, 0, st>>>(P);
         e = cudaGetLastError();
@@ -1186,12 +1135,14 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
     }
     if (e == cudaSuccess && opts && opts->ev_scan_end)
         e = cudaEventRecord((cudaEvent_t)opts->ev_scan_end, st);
-    if (e == cudaSuccess) {
-        k_reduce<<<P.n_chunks ? P.n_chunks : 1, RT, 0, st>>>(P);
+    if (e == cudaSuccess && P.n_tiles && !P.chunk_adds) {
+        k_reduce<<<n_chunks, 256, 0, st>>>(P);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess && P.n_tiles) {
-        k_offsets<<<P.n_chunks, RT, 0, st>>>(P);
+    if (e == cudaSuccess) {
+        // four units per warp where that is all there are (chunks of 32)
+        const uint32_t span = P.chunk_shift == CHUNK_SHIFT_MIN ? 4u : 32u;
+        k_expand<<<n_chunks ? n_chunks : 1, 256, 0, st>>>(P, span);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && opts && opts->ev_emit_begin)
@@ -1222,14 +1173,6 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
     }
     if (e == cudaSuccess && opts && opts->ev_emit_end)
         e = cudaEventRecord((cudaEvent_t)opts->ev_emit_end, st);
-    if (e == cudaSuccess) {
-        const uint64_t maxb = (uint64_t)nsm * 8;
-        const uint32_t span = (uint64_t)P.n_tiles <= maxb * 8 * EXPAND_SPAN_FEW ? EXPAND_SPAN_FEW : EXPAND_SPAN;
-        uint64_t blocks = ((uint64_t)P.n_tiles + 8 * span - 1) / (8 * span);
-        if (blocks > maxb) blocks = maxb;
-        k_expand<<<(uint32_t)(blocks ? blocks : 1), 256, 0, st>>>(P, span);
-        e = cudaGetLastError();
-    }
     if (e != cudaSuccess)
         return set_error(PFAC_ECUDA, "pfac_match: launch failed: %s", cudaGetErrorString(e));
     return PFAC_OK;
