@@ -592,11 +592,7 @@ extern "C" int pfac_build(const uint8_t *const *patterns, const uint32_t *length
         if (!dag && match_density * 512.0 <= 8.0) {
             std::vector<WinPat> wp(n_patterns);
             for (uint32_t i = 0; i < n_patterns; i++) wp[i] = WinPat{pats[order[i]].p, len_at(i)};
-            // the deepest prefix bitmap of at most 64 KiB
-            double dens_f = 1.0;
-            for (uint32_t k = kmin; k <= kmax; k++)
-                if ((1ull << (k * bps)) <= 8ull * 65536)
-                    dens_f = (double)n_ent[k] / (double)(1ull << (k * bps));
+            const double dens_f = (double)n_ent[kmax] / (double)(1ull << (kmax * bps));
             build_window_filter(wp, sigma, bps, std::min(dens_f, 1.0), &wf);
         }
         const uint64_t sz_H = wf.H.size() * 4;

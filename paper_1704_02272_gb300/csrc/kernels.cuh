@@ -122,18 +122,20 @@ struct MatchParams {
     uint32_t dbatch_cap;
     uint2 *dbatch;
     // window kernel: the entry buffer (position << 24 | prefix index), the
-    // filter's split of shared memory and hash, the prefix bitmap of depth
-    // wf_k its candidates are tested against (wf_words of it in shared memory)
+    // filter's split of shared memory and hash, the words of the prefix bitmap
+    // in shared memory (0: its candidates are tested against it through L2)
     uint64_t *wbuf;
-    uint32_t wbuf_cap;
+    uint32_t *wcnt;       // entries of each part of the buffer, WSUB_STRIDE words apart
+    uint32_t wsub_cap;    // entries a part holds
+    uint32_t wsub_mask;   // parts - 1 (a power of two, at most WSUB_MAX parts)
     uint32_t w_words, w_rep, w_gm, w_glen;
     uint32_t w_badmask;   // byte bits outside the symbol range, where they matter to the filter
-    const uint32_t *wf;
-    uint32_t wf_words, wf_k;
+    uint32_t wf_words;
     uint32_t unordered;  // a unit's records are in no order (the expansion sorts them)
 };
 
 constexpr uint32_t UNIT_NONE = 0xFFFFFFFFu;
+constexpr uint32_t WSUB_MAX = 64, WSUB_STRIDE = 32;
 // a unit's keys fit: 512 positions of at most 2^24 ids each
 constexpr int UNIT_KEY_BITS = 40;
 

@@ -20,8 +20,9 @@
 //   full queue is flushed by all lanes: the prefix index of each start is
 //   packed from the text (still in L2), tested against a prefix bitmap in
 //   shared memory (or through L2) and the passing starts are appended to the
-//   call's entry buffer with one atomic.  When the buffer is full the lanes
-//   walk their starts from the root instead.
+//   call's entry buffer with one atomic, on one of up to 64 parts of it so
+//   that the warps do not queue on one counter.  When a part is full its
+//   warps' lanes walk their starts from the root instead.
 // * k_wresolve then takes the entries in any order: segment limit, exact
 //   prefix bit, the batched walks of the queued kernel's resolver, and one
 //   record per match at an atomically taken slot of its slice; the key
@@ -196,19 +197,21 @@ __device__ __forceinline__ uint32_t w_walk_fin(const MatchParams &P, uint64_t ub
     }
 }
 
+__device__ __forceinline__ uint32_t w_walk_any(const MatchParams &P, uint64_t ub, uint32_t pos,
+                                               uint32_t lim) {
+    switch (P.T.W) {
+        case 0: return w_walk_fin<0>(P, ub, pos, lim);
+        case 1: return w_walk_fin<1>(P, ub, pos, lim);
+        case 2: return w_walk_fin<2>(P, ub, pos, lim);
+        case 3: return w_walk_fin<3>(P, ub, pos, lim);
+        default: return w_walk_fin<8>(P, ub, pos, lim);
+    }
+}
+
 static __device__ __noinline__ void w_walk(const MatchParams *PP, uint64_t p) {
     const MatchParams &P = *PP;
     const uint32_t u = (uint32_t)(p >> SLICE_SHIFT), pos = (uint32_t)p & (SLICE - 1);
-    const uint32_t lim = w_limit(P, u, p);
-    const uint64_t ub = (uint64_t)u << SLICE_SHIFT;
-    uint32_t fin = 0;
-    switch (P.T.W) {
-        case 0: fin = w_walk_fin<0>(P, ub, pos, lim); break;
-        case 1: fin = w_walk_fin<1>(P, ub, pos, lim); break;
-        case 2: fin = w_walk_fin<2>(P, ub, pos, lim); break;
-        case 3: fin = w_walk_fin<3>(P, ub, pos, lim); break;
-        default: fin = w_walk_fin<8>(P, ub, pos, lim); break;
-    }
+    const uint32_t fin = w_walk_any(P, (uint64_t)u << SLICE_SHIFT, pos, w_limit(P, u, p));
     if (fin) w_emit(P, u, pos, fin);
 }
 
@@ -269,12 +272,10 @@ __device__ __forceinline__ uint32_t w_prefix(const MatchParams &P, const WText<P
 // survivors go to the entry buffer (position << 24 | prefix index), or are
 // walked here when it is full.
 template <int PACKED, int S>
-__device__ __noinline__ void w_flush(const MatchParams *PP, const uint32_t *q, uint32_t n,
-                                     const uint32_t *Fs, uint32_t gw, uint32_t gstride,
-                                     uint32_t lane) {
-    const MatchParams &P = *PP;
+__device__ __forceinline__ void w_flush(const MatchParams &P, const uint32_t *q, uint32_t n,
+                                        const uint32_t *Fs, uint32_t gw, uint32_t gstride,
+                                        uint32_t lane) {
     const uint32_t lt = (1u << lane) - 1u;
-    const uint32_t f_mask = (1u << (P.wf_k * P.T.bps)) - 1u;
     constexpr int R = PACKED ? 2 : 4;  // rounds of 32 starts whose loads overlap
     for (uint32_t e0 = 0; e0 < n * S; e0 += 32 * R) {
         uint64_t en[R];
@@ -295,8 +296,8 @@ __device__ __noinline__ void w_flush(const MatchParams *PP, const uint32_t *q, u
         for (int r = 0; r < R; r++) {
             const uint64_t p = en[r];
             const uint32_t x = w_prefix<PACKED>(P, tx[r], p);
-            const uint32_t fx = x & f_mask;
-            const uint32_t fw = Fs ? Fs[fx >> 5] : __ldg(P.wf + (fx >> 5));
+            const uint32_t fx = x == WX_ROOT ? 0u : (uint32_t)chk(P, x, 1ull << (P.k * P.T.bps));
+            const uint32_t fw = Fs ? Fs[fx >> 5] : __ldg(P.F + (fx >> 5));
             const bool keep = p != ~0ull && (x == WX_ROOT || ((fw >> (fx & 31)) & 1u));
             en[r] = (p << 24) | x;
             kept[r] = __ballot_sync(0xFFFFFFFFu, keep);
@@ -305,17 +306,19 @@ __device__ __noinline__ void w_flush(const MatchParams *PP, const uint32_t *q, u
 #pragma unroll
         for (int r = 0; r < R; r++) tot += __popc(kept[r]);
         if (tot == 0) continue;
-        // no reservation once the buffer is full, so that the counter stays
-        // within one reservation per warp of its capacity
-        uint32_t base = P.wbuf_cap;
-        if (lane == 0 && *(volatile uint32_t *)&P.hdr->defer_entries < P.wbuf_cap)
-            base = atomicAdd(&P.hdr->defer_entries, tot);
+        // the warp's part of the buffer; no reservation once it is full, so
+        // that its counter stays within one reservation per warp of its size
+        const uint32_t sub = gw & P.wsub_mask;
+        uint32_t *cnt = P.wcnt + sub * WSUB_STRIDE;
+        uint64_t *buf = P.wbuf + (size_t)sub * P.wsub_cap;
+        uint32_t base = P.wsub_cap;
+        if (lane == 0 && *(volatile uint32_t *)cnt < P.wsub_cap) base = atomicAdd(cnt, tot);
         base = __shfl_sync(0xFFFFFFFFu, base, 0);
 #pragma unroll
         for (int r = 0; r < R; r++) {
             if ((kept[r] >> lane) & 1u) {
                 const uint32_t at = base + __popc(kept[r] & lt);
-                if (at < P.wbuf_cap) P.wbuf[at] = en[r];
+                if (at < P.wsub_cap) buf[at] = en[r];
                 else w_walk(&P, en[r] >> 24);
             }
             base += __popc(kept[r]);
@@ -388,7 +391,7 @@ __global__ void __launch_bounds__((TB == WT_L2 ? WNW_SMALL : WNW) * 32, 1)
     if (TB != WT_L2) {
         w_fill<NW * 32>(reinterpret_cast<uint32_t *>(smem), P.T.H, P.w_words,
                         TB == WT_ONE ? 0u : P.w_rep, blockIdx.x * 160u);
-        w_fill<NW * 32>(Fs, P.wf, P.wf_words, 0u, blockIdx.x * 32u);
+        w_fill<NW * 32>(Fs, P.F, P.wf_words, 0u, blockIdx.x * 32u);
         __syncthreads();
     }
     WConst K;
@@ -403,158 +406,375 @@ __global__ void __launch_bounds__((TB == WT_L2 ? WNW_SMALL : WNW) * 32, 1)
     const uint32_t lt = (1u << lane) - 1u;
     const bool l31 = lane == 31;
     const bool al32 = ((uintptr_t)P.in & 31) == 0;
-    uint32_t qn = 0;
     auto load_head = [&](bool on, const uint8_t *a) -> uint4 {
         if (!PACKED) return make_uint4(ld_stream4_if(on, a), 0u, 0u, 0u);
         return ld_stream16_if(on, a);
     };
-    // one step: the warp's i-th chunk of 1,024 bytes from registers (h: the
-    // next chunk's head, on lane 31); forced = windows that are candidates
-    // whatever the filter says
-    auto step = [&](uint32_t i, const WChunk &c, const uint4 &h, uint32_t forced) {
-        uint32_t w[9];
-        if (!PACKED) {
-#pragma unroll
-            for (int x = 0; x < 8; x++) w[x] = c.w[x];
-            const uint32_t nx = __shfl_down_sync(0xFFFFFFFFu, c.w[0], 1);
-            w[8] = l31 ? h.x : nx;
-        } else {
-            w[0] = r_pack2(make_uint4(c.w[0], c.w[1], c.w[2], c.w[3]));
-            w[1] = r_pack2(make_uint4(c.w[4], c.w[5], c.w[6], c.w[7]));
-            // lane 31 offers the next chunk's head to itself
-            const uint32_t nx = __shfl_down_sync(0xFFFFFFFFu, w[0], 1);
-            w[2] = l31 ? r_pack2(h) : nx;
-#pragma unroll
-            for (int x = 3; x < 9; x++) w[x] = 0;
+    // clean chunks: every load, the next chunk's head included, inside the input
+    const uint64_t gc = N >= HALO ? (N - HALO) >> (SLICE_SHIFT + 1) : 0;
+    const uint32_t g_clean = gc < n_pairs ? (uint32_t)gc : n_pairs;
+    const uint32_t n_it = (n_pairs - gw + gstride - 1) / gstride;  // gw < n_pairs or no step
+    const uint32_t n_ok = gw < g_clean ? (g_clean - gw + gstride - 1) / gstride : 0u;
+    const uint64_t step_b = (uint64_t)gstride << (SLICE_SHIFT + 1);
+    const uint8_t *src = P.in + ((uint64_t)gw << (SLICE_SHIFT + 1)) + lane * 32u;
+    // the warp's i-th chunk and, on lane 31, the head of the chunk after it;
+    // past the clean ones as far as the input goes in whole 16-byte pieces
+    auto load = [&](uint32_t i, WChunk &c, uint4 &h) {
+        if (i < n_ok) {
+            w_load32(src, al32, c);
+            h = load_head(l31, src + 32);
+            return;
         }
-        uint32_t m = w_filter<PACKED, S, NB, G5, TB>(w, K) | forced;
-        if (P.w_badmask) {
-            // bytes outside the packed symbol range, where H would need
-            // completions over them (patterns that end inside a window): the
-            // windows that may hold one are candidates (all of a lane's, in
-            // the rare steps that have any)
-            const uint32_t hm = P.w_badmask;
-            const uint32_t ra = (c.w[0] | c.w[1] | c.w[2] | c.w[3] | c.w[4] | c.w[5] | c.w[6] | c.w[7]) & hm;
-            const uint32_t rh = (h.x | h.y | h.z | h.w) & hm;
-            if (__any_sync(0xFFFFFFFFu, (ra | rh) != 0)) {
-                const uint32_t na = __ballot_sync(0xFFFFFFFFu, ra != 0);
-                const uint32_t nh = __ballot_sync(0xFFFFFFFFu, rh != 0);
-                if (((na >> lane) & 1u) || (l31 ? nh != 0 : ((na >> (lane + 1)) & 1u)))
-                    m |= NWIN == 32 ? 0xFFFFFFFFu : (1u << (NWIN & 31)) - 1u;
+        const uint64_t s0 = (gw + (uint64_t)i * gstride) << (SLICE_SHIFT + 1), o = s0 + lane * 32u;
+        const uint4 a = ld_stream16_if(o + 16 <= N, P.in + o);
+        const uint4 b = ld_stream16_if(o + 32 <= N, P.in + o + 16);
+        c = WChunk{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
+        h = load_head(l31 && s0 + 2 * SLICE + HALO <= N, P.in + s0 + 2 * SLICE);
+    };
+    WChunk c0, c1;
+    uint4 h0, h1;
+    uint32_t qn = 0;
+    if (gw >= n_pairs) return;
+    for (uint32_t f = 1; f < WPF && f < n_ok; f++)
+        prefetch_l2_if(lane == 0, src + f * step_b, 2 * SLICE);
+    load(0, c0, h0);
+    for (uint32_t i = 0;; i++) {
+        src += step_b;
+        prefetch_l2_if(lane == 0 && i + WPF < n_ok, src + (WPF - 1) * step_b, 2 * SLICE);
+        if (i + 1 < n_it) load(i + 1, c1, h1);
+        uint32_t m = 0;
+        if (i < n_it) {
+            uint32_t w[9];
+            if (!PACKED) {
+#pragma unroll
+                for (int x = 0; x < 8; x++) w[x] = c0.w[x];
+                const uint32_t nx = __shfl_down_sync(0xFFFFFFFFu, c0.w[0], 1);
+                w[8] = l31 ? h0.x : nx;
+            } else {
+                w[0] = r_pack2(make_uint4(c0.w[0], c0.w[1], c0.w[2], c0.w[3]));
+                w[1] = r_pack2(make_uint4(c0.w[4], c0.w[5], c0.w[6], c0.w[7]));
+                const uint32_t nx = __shfl_down_sync(0xFFFFFFFFu, w[0], 1);
+                w[2] = l31 ? r_pack2(h0) : nx;
+#pragma unroll
+                for (int x = 3; x < 9; x++) w[x] = 0;
+            }
+            m = w_filter<PACKED, S, NB, G5, TB>(w, K);
+            if (P.w_badmask) {
+                // bytes outside the packed symbol range, where H would need
+                // completions over them (patterns that end inside a window):
+                // the windows that may hold one are candidates (all of a
+                // lane's, in the rare steps that have any)
+                const uint32_t hm = P.w_badmask;
+                const uint32_t ra = (c0.w[0] | c0.w[1] | c0.w[2] | c0.w[3] | c0.w[4] | c0.w[5] |
+                                     c0.w[6] | c0.w[7]) & hm;
+                const uint32_t rh = (h0.x | h0.y | h0.z | h0.w) & hm;
+                if (__any_sync(0xFFFFFFFFu, (ra | rh) != 0)) {
+                    const uint32_t na = __ballot_sync(0xFFFFFFFFu, ra != 0);
+                    const uint32_t nh = __ballot_sync(0xFFFFFFFFu, rh != 0);
+                    if (((na >> lane) & 1u) || (l31 ? nh != 0 : ((na >> (lane + 1)) & 1u)))
+                        m |= NWIN == 32 ? 0xFFFFFFFFu : (1u << (NWIN & 31)) - 1u;
+                }
+            }
+            if (i >= n_ok) {
+                // windows that reach past the whole 16-byte pieces are
+                // candidates (starts at or past starts_end are dropped by
+                // the flush)
+                const uint64_t o = ((gw + (uint64_t)i * gstride) << (SLICE_SHIFT + 1)) + lane * 32u;
+                for (uint32_t x = 0; x < NWIN; x++)
+                    if (o + x * S + S - 1 + P.w_glen > N16) m |= 1u << x;
             }
         }
+        // candidates to the queue, a round per lane's next one; a full queue
+        // is flushed, and after the last chunk what is left
         uint32_t any = __ballot_sync(0xFFFFFFFFu, m != 0);
-        while (any) {
+        while (any || (i >= n_it && qn)) {
             if (m) {
                 const uint32_t j = __ffs(m) - 1;
                 m &= m - 1;
                 q[qn + __popc(any & lt)] = (i << 10) + (lane * 32 + j * S + S - 1);
             }
             qn += __popc(any);
-            if (qn > WQCAP - 32) {
+            if (qn > WQCAP - 32 || i >= n_it) {
                 __syncwarp();
-                w_flush<PACKED, S>(&P, q, qn, Fq, gw, gstride, lane);
+                w_flush<PACKED, S>(P, q, qn, Fq, gw, gstride, lane);
                 qn = 0;
             }
             any = __ballot_sync(0xFFFFFFFFu, m != 0);
         }
-    };
-    // clean chunks: every load, the next chunk's head included, inside the input
-    const uint64_t gc = N >= HALO ? (N - HALO) >> (SLICE_SHIFT + 1) : 0;
-    const uint32_t g_clean = gc < n_pairs ? (uint32_t)gc : n_pairs;
-    const uint32_t n_it = gw < g_clean ? (g_clean - gw + gstride - 1) / gstride : 0u;
-    const uint64_t step_b = (uint64_t)gstride << (SLICE_SHIFT + 1);
-    const uint8_t *src = P.in + ((uint64_t)gw << (SLICE_SHIFT + 1)) + lane * 32u;
-    uint32_t i = 0;
-    if (n_it) {
-        for (uint32_t f = 1; f < WPF && f < n_it; f++)
-            prefetch_l2_if(lane == 0, src + f * step_b, 2 * SLICE);
-        WChunk c0, c1;
-        uint4 h0, h1;
-        w_load32(src, al32, c0);
-        h0 = load_head(l31, src + 32);
-        for (;; i++) {
-            const bool more = i + 1 < n_it;
-            src += step_b;
-            if (WPF) prefetch_l2_if(lane == 0 && i + WPF < n_it, src + (WPF - 1) * step_b, 2 * SLICE);
-            if (more) {
-                w_load32(src, al32, c1);
-                h1 = load_head(l31, src + 32);
-            }
-            step(i, c0, h0, 0u);
-            if (!more) break;
-            c0 = c1;
-            h0 = h1;
-        }
-        i++;
-    }
-    // the last chunks: loads as far as the input goes in whole 16-byte pieces;
-    // windows that reach past them are candidates (starts at or past
-    // starts_end are dropped by the flush)
-    for (uint32_t g = gw + i * gstride; g < n_pairs; g += gstride, i++) {
-        const uint64_t s0 = (uint64_t)g << (SLICE_SHIFT + 1), o = s0 + lane * 32u;
-        uint4 a = make_uint4(0, 0, 0, 0), b = a;
-        if (o + 16 <= N) a = ld_stream16(P.in + o);
-        if (o + 32 <= N) b = ld_stream16(P.in + o + 16);
-        const WChunk c{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
-        const uint4 h = load_head(l31 && s0 + 2 * SLICE + HALO <= N, P.in + s0 + 2 * SLICE);
-        uint32_t forced = 0;
-        for (uint32_t x = 0; x < NWIN; x++)
-            if (o + x * S + S - 1 + P.w_glen > N16) forced |= 1u << x;
-        step(i, c, h, forced);
-    }
-    if (qn) {
-        __syncwarp();
-        w_flush<PACKED, S>(&P, q, qn, Fq, gw, gstride, lane);
+        if (i >= n_it) break;
+        c0 = c1;
+        h0 = h1;
     }
 }
 
-// Resolves the entries the scan left: each warp takes blocks of up to 128.
-template <int W>
+// Resolves the entries the scan left: each warp takes blocks of up to 64, two
+// per lane.  What bounds it is the chain of dependent L2 loads of a walk, so
+// the loads that do not depend on each other go out together: the slice's
+// first offset indices and the eight symbols after the prefix, then the prefix
+// node's words and the segment end, the prefix entry, and one record a round
+// with the symbols at hand.  Walks still running after three rounds
+// are packed one per lane and advance up to eight records of a chain at a
+// time.
+constexpr int WRU = 2;                       // entries per lane
+constexpr uint32_t WRB = 32 * WRU;           // and per block
+struct WTail {
+    uint32_t unit[WRB], pos[WRB], q[WRB], lim[WRB], state[WRB], slot[WRB];
+};
+// pending records of the dense scan kernel (kernels_d.cuh): an entry is the
+// record's index, its output word holds the state to walk from
+constexpr uint32_t D_PEND = 0x80000000u, D_PEND_ROOT = 0x40000000u, D_PEND_STATE = 0x3FFFFFFFu;
+
+// A resolved walk's output: a match of the window kernel, or the pending
+// record's output (0: none) and its keys.
+template <int DENSE>
+__device__ __forceinline__ void w_result(const MatchParams &P, uint32_t u, uint32_t pos, uint32_t slot,
+                                         uint32_t fin) {
+    if (!DENSE) {
+        if (fin) w_emit(P, u, pos, fin);
+        return;
+    }
+    P.recs[(size_t)u * P.unit_cap + slot] = ((uint64_t)pos << 32) | fin;
+    if (fin) atomicAdd((unsigned long long *)(P.tile_k + u), (unsigned long long)fin_len_c(P, fin));
+}
+
+template <int W, int DENSE>
 __global__ void __launch_bounds__(RES_WARPS * 32, RES_CTAS)
     k_wresolve(const __grid_constant__ MatchParams P) {
-    __shared__ RWarpArea areas[RES_WARPS];
+    __shared__ WTail tails[RES_WARPS];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
-    RWarpArea &A = areas[warp];
-    const uint32_t n0 = *(volatile uint32_t *)&P.hdr->defer_entries;
-    const uint32_t n = n0 < P.wbuf_cap ? n0 : P.wbuf_cap;
+    WTail &T = tails[warp];
     const uint32_t gw = blockIdx.x * RES_WARPS + warp, gs = gridDim.x * RES_WARPS;
-    // few entries: 32 at a time, so that more warps share the latency
-    const uint32_t blk = n > gs * QCAP ? (uint32_t)QCAP : 32u;
-    const uint32_t k = P.k;
-    for (uint64_t b = (uint64_t)gw * blk; b < n; b += (uint64_t)gs * blk) {
-        uint32_t qn = 0;
-        for (uint32_t r = 0; r < blk; r += 32) {
-            const uint64_t e = b + r + lane;
-            bool keep = false;
-            QEntry en{0u, 0u, 0u, 0u};
-            if (e < n) {
-                const uint64_t v = P.wbuf[e];
+    // the buffer's parts: lane l counts those of parts l and l + 32
+    const uint32_t parts = P.wsub_mask + 1;
+    uint32_t n0 = lane < parts ? *(volatile uint32_t *)(P.wcnt + lane * WSUB_STRIDE) : 0u;
+    uint32_t n1 = lane + 32 < parts ? *(volatile uint32_t *)(P.wcnt + (lane + 32) * WSUB_STRIDE) : 0u;
+    n0 = n0 < P.wsub_cap ? n0 : P.wsub_cap;
+    n1 = n1 < P.wsub_cap ? n1 : P.wsub_cap;
+    // few entries: blocks of 32, so that more warps share the latency
+    const uint32_t all = __reduce_add_sync(0xFFFFFFFFu, (n0 + 31) / 32 + (n1 + 31) / 32);
+    const uint32_t blk = all > gs ? WRB : 32u;
+    // blocks up to and including each part
+    uint32_t i0 = (n0 + blk - 1) / blk, i1 = (n1 + blk - 1) / blk;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t a = __shfl_up_sync(0xFFFFFFFFu, i0, o), c = __shfl_up_sync(0xFFFFFFFFu, i1, o);
+        if (lane >= (uint32_t)o) {
+            i0 += a;
+            i1 += c;
+        }
+    }
+    i1 += __shfl_sync(0xFFFFFFFFu, i0, 31);
+    const uint32_t n_blk = __shfl_sync(0xFFFFFFFFu, i1, 31);
+
+    const uint32_t k = P.k, sigma = P.T.sigma, psh = W == 3 ? sigma : P.T.pk_shift;
+    const uint32_t bmask = W == 0 ? (1u << psh) - 1u : META_BASE_MASK;
+    const uint32_t *__restrict__ rec = P.T.rec;
+    for (uint32_t bi = gw; bi < n_blk; bi += gs) {
+        // the block's part, its place there and the part's entries
+        const uint32_t sub = __popc(__ballot_sync(0xFFFFFFFFu, i0 <= bi)) +
+                             __popc(__ballot_sync(0xFFFFFFFFu, i1 <= bi));
+        const uint32_t e0 = __shfl_sync(0xFFFFFFFFu, i0, (sub - 1) & 31);
+        const uint32_t e1 = __shfl_sync(0xFFFFFFFFu, i1, (sub - 1) & 31);
+        const uint32_t before = sub == 0 ? 0u : (sub <= 32 ? e0 : e1);
+        const uint32_t s0 = __shfl_sync(0xFFFFFFFFu, n0, sub & 31);
+        const uint32_t s1 = __shfl_sync(0xFFFFFFFFu, n1, sub & 31);
+        const uint32_t n = sub < 32 ? s0 : s1;
+        const uint64_t *buf = P.wbuf + (size_t)sub * P.wsub_cap;
+        const uint32_t b = (bi - before) * blk;
+
+        // ---- prefix entry, walk limit and the symbols after the prefix
+        // state: -1 nothing to do, 0 walking from st at q, 1 stopped at st,
+        // 2 stopped on merged leaf st, 3 output known (fin)
+        int state[WRU];
+        uint32_t unit[WRU], pos[WRU], lim[WRU], st[WRU], q[WRU], fin[WRU], tq[WRU], t0[WRU], t1[WRU];
+        uint32_t slo[WRU], shi[WRU], x[WRU], slot[WRU];
+#pragma unroll
+        for (int u = 0; u < WRU; u++) {
+            const uint32_t e = b + 32 * u + lane;
+            const bool on = e < n && (uint32_t)(32 * u) < blk;
+            const uint64_t v = on ? buf[e] : 0ull;
+            state[u] = on ? 0 : -1;
+            st[u] = 0;
+            if (DENSE) {
+                const uint64_t r = on ? P.recs[v] : 0ull;
+                unit[u] = (uint32_t)chk(P, v >> SLICE_SHIFT, P.n_tiles ? P.n_tiles : 1);
+                slot[u] = (uint32_t)v & (SLICE - 1);
+                pos[u] = (uint32_t)(r >> 32);
+                st[u] = (uint32_t)r & D_PEND_STATE;
+                x[u] = (uint32_t)r & D_PEND_ROOT ? WX_ROOT : 0u;
+            } else {
                 const uint64_t p = v >> 24;
-                const uint32_t x = (uint32_t)v & 0xFFFFFFu;
-                en.unit = (uint32_t)chk(P, p >> SLICE_SHIFT, P.n_tiles);
-                en.pos = (uint32_t)p & (SLICE - 1);
-                en.lim = w_limit(P, en.unit, p);
-                en.x = x;
-                keep = true;
-                if (x == WX_ROOT || en.pos + k > en.lim) {
-                    en.x = ROOT_X;
+                unit[u] = (uint32_t)chk(P, p >> SLICE_SHIFT, P.n_tiles ? P.n_tiles : 1);
+                slot[u] = 0;
+                pos[u] = (uint32_t)p & (SLICE - 1);
+                x[u] = (uint32_t)v & 0xFFFFFFu;
+            }
+            // the slice's first offset indices, the text from p + k on (from
+            // p for a walk from the root)
+            slo[u] = shi[u] = 0;
+            if (P.n_seg > 1) {
+                slo[u] = __ldg(P.unit_seg + unit[u]);
+                shi[u] = unit[u] + 1 < P.n_tiles ? __ldg(P.unit_seg + unit[u] + 1) : P.n_seg;
+            }
+            tq[u] = pos[u] + (x[u] == WX_ROOT ? 0u : k);
+            const uint64_t a = ((uint64_t)unit[u] << SLICE_SHIFT) + tq[u], c = a & ~3ull;
+            const bool ok = on && c + 12 <= P.n;
+            const uint8_t *src = P.in + (ok ? c : 0ull);
+            const uint32_t w0 = ld_stream4_if(ok, src), w1 = ld_stream4_if(ok, src + 4),
+                           w2 = ld_stream4_if(ok, src + 8);
+            const uint32_t sh = 8 * ((uint32_t)a & 3u);
+            t0[u] = __funnelshift_r(w0, w1, sh);
+            t1[u] = __funnelshift_r(w1, w2, sh);
+            if (!ok) tq[u] = 0xFFFFFF00u;  // no symbol at hand
+        }
+#pragma unroll
+        for (int u = 0; u < WRU; u++) {
+            const uint64_t us = (uint64_t)unit[u] << SLICE_SHIFT, p = us + pos[u];
+            const uint64_t remain = P.n - us;
+            lim[u] = remain < LIM_MAX ? (uint32_t)remain : LIM_MAX;
+            if (P.n_seg > 1) {
+                // (bounded: offsets out of order leave some indices unwritten)
+                uint32_t lo = slo[u] < P.n_seg ? slo[u] : P.n_seg, hi = shi[u] < P.n_seg ? shi[u] : P.n_seg;
+                while (lo < hi) {
+                    const uint32_t mid = (lo + hi) >> 1;
+                    if (__ldg(P.seg + mid) > p) hi = mid; else lo = mid + 1;
+                }
+                const uint64_t e = __ldg(P.seg + lo);
+                const uint64_t r = e > us ? e - us : 0;
+                lim[u] = r < lim[u] ? (uint32_t)r : lim[u];
+            }
+            fin[u] = 0;
+            q[u] = pos[u];
+            if (DENSE) {
+                if (x[u] != WX_ROOT) q[u] += k;
+            } else if (state[u] == 0 && x[u] != WX_ROOT && pos[u] + k <= lim[u]) {
+                // (the scan has tested the index's bit)
+                const uint32_t xx = (uint32_t)chk(P, x[u], 1ull << (k * P.T.bps));
+                const uint32_t r = (uint32_t)chk(P, prefix_rank(P.F, 0, P.C, P.c_shift, xx), P.T.n_e[k]);
+                const uint32_t ev = __ldg(P.E + r);
+                q[u] = pos[u] + k;
+                if (ev & D_CONT) {
+                    st[u] = ev & D_VAL_MASK;
                 } else {
-                    const uint32_t xx = (uint32_t)chk(P, x, 1ull << (k * P.T.bps));
-                    keep = ((__ldg(P.F + (xx >> 5)) >> (xx & 31)) & 1u) != 0;
+                    state[u] = 3;
+                    fin[u] = ev;
                 }
             }
-            const uint32_t bm = __ballot_sync(0xFFFFFFFFu, keep);
-            if (keep) A.q[qn + __popc(bm & lt)] = en;
-            qn += __popc(bm);
+        }
+        // symbol at slice offset i of walk u
+        auto symbol = [&](int u, uint32_t i) -> uint32_t {
+            if (i >= lim[u]) return 0x100u;
+            const uint32_t d = i - tq[u];
+            if (d < 8) return ((d < 4 ? t0[u] : t1[u]) >> (8 * (d & 3))) & 0xFFu;
+            return __ldg(P.in + chk(P, ((uint64_t)unit[u] << SLICE_SHIFT) + i, P.n));
+        };
+        // ---- three rounds, one record of each walk a round
+#pragma unroll 1
+        for (int round = 0; round < 3; round++) {
+            bool any = false;
+#pragma unroll
+            for (int u = 0; u < WRU; u++) any |= state[u] == 0;
+            if (!__any_sync(0xFFFFFFFFu, any)) break;
+            uint32_t c[WRU], wd[WRU], bl[WRU], mt[WRU], f1[WRU];
+#pragma unroll
+            for (int u = 0; u < WRU; u++) {
+                if (state[u] != 0) continue;
+                c[u] = symbol(u, q[u]);
+                load_step<W>(rec, (uint32_t)chk(P, st[u], P.T.n_rec), c[u], wd[u], bl[u], mt[u], f1[u], psh);
+            }
+#pragma unroll
+            for (int u = 0; u < WRU; u++) {
+                if (state[u] != 0) continue;
+                const uint32_t cur = st[u];
+                const int r = take_step(sigma, c[u], wd[u], bl[u], mt[u], st[u], bmask);
+                if (r == 0) {
+                    q[u]++;
+                } else if (r == 2) {
+                    state[u] = 2;
+                } else if (W == 0 && !(mt[u] & PK_FIN)) {
+                    state[u] = 3;
+                } else if (W <= 1 || W == 3) {  // outputs in their own array
+                    st[u] = cur;
+                    state[u] = 1;
+                } else {
+                    fin[u] = f1[u];
+                    state[u] = 3;
+                }
+            }
+        }
+        // ---- the walks still running, one per lane
+        uint32_t nt = 0;
+#pragma unroll
+        for (int u = 0; u < WRU; u++) {
+            const bool w = state[u] == 0;
+            const uint32_t bm = __ballot_sync(0xFFFFFFFFu, w);
+            if (w) {
+                const uint32_t t = nt + __popc(bm & lt);
+                T.unit[t] = unit[u];
+                T.pos[t] = pos[u];
+                T.q[t] = q[u];
+                T.lim[t] = lim[u];
+                T.state[t] = st[u];
+                T.slot[t] = slot[u];
+            }
+            nt += __popc(bm);
         }
         __syncwarp();
-        if (qn == 0) continue;
-        resolve_batch_inl<W, VAR_F | VAR_RES>(P, A.q, qn, P.F, P.C, nullptr, lane);
-        for (uint32_t e = lane; e < qn; e += 32) {
-            const QEntry en = A.q[e];
-            if (en.x) w_emit(P, en.unit, en.pos, en.x);
+        // outputs of the walks that have stopped
+#pragma unroll
+        for (int u = 0; u < WRU; u++) {
+            if (state[u] == 1) fin[u] = rec_fin<W>(P, st[u], 0, PK_FIN);
+            else if (state[u] == 2) fin[u] = __ldg(P.T.leaf_fin + chk(P, st[u], P.T.leaf_words));
+            if (state[u] >= 1) w_result<DENSE>(P, unit[u], pos[u], slot[u], fin[u]);
+        }
+        for (uint32_t b0 = 0; b0 < nt; b0 += 32) {
+            const uint32_t t = b0 + lane;
+            if (t < nt) {
+                const uint32_t un = T.unit[t], lm = T.lim[t];
+                uint32_t s1 = T.state[t], q1 = T.q[t], f = 0;
+                const uint64_t ub = (uint64_t)un << SLICE_SHIFT;
+                // each round fetches TS consecutive records from the current
+                // state and the next TS symbols; along a single-child chain
+                // (placed in consecutive records) it advances up to TS levels
+                constexpr int TS = (W == 8 || W == 2) ? 4 : 8;
+                const uint32_t n_rec = P.T.n_rec;
+                bool done = false;
+                while (!done) {
+                    uint32_t c[TS], wd[TS], bl[TS], mt[TS], f1[TS];
+#pragma unroll
+                    for (int i = 0; i < TS; i++) {
+                        c[i] = q1 + i < lm ? (uint32_t)__ldg(P.in + chk(P, ub + q1 + i, P.n)) : 0x100u;
+                        if (i == 0 || s1 + i < n_rec) {
+                            load_step<W>(rec, (uint32_t)chk(P, s1 + i, n_rec), c[i], wd[i], bl[i], mt[i],
+                                         f1[i], psh);
+                        } else {
+                            wd[i] = bl[i] = mt[i] = f1[i] = 0;
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < TS; i++) {
+                        uint32_t nx = 0;
+                        const uint32_t cur = s1 + i;
+                        const int r = take_step(sigma, c[i], wd[i], bl[i], mt[i], nx, bmask);
+                        if (r == 1) {
+                            f = rec_fin<W>(P, cur, f1[i], mt[i]);
+                            done = true;
+                            break;
+                        }
+                        if (r == 2) {
+                            f = __ldg(P.T.leaf_fin + chk(P, nx, P.T.leaf_words));
+                            done = true;
+                            break;
+                        }
+                        if (i + 1 < TS && nx == cur + 1) continue;
+                        s1 = nx;
+                        q1 += i + 1;
+                        break;
+                    }
+                }
+                w_result<DENSE>(P, un, T.pos[t], T.slot[t], f);
+            }
         }
         __syncwarp();
     }

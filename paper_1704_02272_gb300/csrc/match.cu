@@ -6,10 +6,11 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "internal.h"
-#include "kernels_w.cuh"
+#include "kernels_d.cuh"
 
 namespace pfac {
 
@@ -33,6 +34,8 @@ void *scan_kernel_r2_g1_fe(int rep, int nw);
 
 void *resolve_kernel(int w);
 void *wresolve_kernel(int w);
+void *dresolve_kernel(int w);
+void *scan_kernel_d(bool entries_in_smem);
 void *scan_kernel_w1(bool packed, uint32_t nb, bool g5, int tb);
 void *scan_kernel_w2(bool packed, uint32_t nb, bool g5, int tb);
 void *scan_kernel_w4(bool packed, uint32_t nb, bool g5, int tb);
@@ -172,8 +175,8 @@ __global__ void __launch_bounds__(256) k_reduce(const MatchParams P) {
 // Output offsets and keys of one chunk of units per CTA; the last chunk's CTA
 // writes the total count.  A CTA adds up the counts of the chunks before its
 // own (at most CHUNKS_MAX) and scans its units' counts 8 * span at a time:
-// `span` consecutive units per warp, 32, or 4 when there are few, so that the
-// chains of dependent loads run in more warps.  Units whose records were not
+// `span` consecutive units per warp, 32, or fewer in small chunks, so that the
+// chains of dependent loads run in every warp.  Units whose records were not
 // kept get their offset stored for the emit pass.
 //
 // A warp deals its units that have records out to groups of eight lanes, one record a lane: four units at a
@@ -241,43 +244,58 @@ __global__ void __launch_bounds__(256) k_expand(const MatchParams P, const uint3
         if (ml > P.unit_cap) P.key_off[tl] = ol;
         uint32_t few = __ballot_sync(0xFFFFFFFFu, ml != 0 && ml <= EXPAND_GROUP);
         uint32_t many = __ballot_sync(0xFFFFFFFFu, ml > EXPAND_GROUP && ml <= P.unit_cap);
-        while (few) {
+        // the records of the next four units are loaded while the keys of
+        // the current four are written
+        uint32_t jn = 0;
+        uint64_t rn = 0, on = 0;
+        auto next_few = [&]() {
             // the group's unit: the grp-th set bit
             uint32_t f = few;
             for (uint32_t x = 0; x < grp; x++) f &= f - 1;
-            const uint32_t j = f ? __ffs(f) - 1 : 0u;
-            const uint32_t m = __shfl_sync(0xFFFFFFFFu, ml, j);
-            const uint64_t o = __shfl_sync(0xFFFFFFFFu, ol, j);
-            uint64_t r = 0;
-            uint32_t L = 0;
-            if (f && gl < m) {
-                r = P.recs[(t0 + j) * P.unit_cap + gl];
-                L = fin_len_c(P, (uint32_t)r);
-            }
-            const uint32_t before = keys_before<EXPAND_GROUP>((uint32_t)(r >> 32), L, un, lane);
-            write_keys(P, r, L, t0 + j, o + before);
+            jn = f ? __ffs(f) - 1 : 0u;
+            const uint32_t m = __shfl_sync(0xFFFFFFFFu, ml, jn);
+            on = __shfl_sync(0xFFFFFFFFu, ol, jn);
+            rn = f && gl < m ? P.recs[(t0 + jn) * P.unit_cap + gl] : 0ull;
 #pragma unroll
             for (uint32_t x = 0; x < 32 / EXPAND_GROUP; x++) few &= few - 1;
+        };
+        bool more = few != 0;
+        if (more) next_few();
+        while (more) {
+            const uint64_t r = rn, o = on, t = t0 + jn;
+            more = few != 0;
+            if (more) next_few();
+            const uint32_t L = (uint32_t)r ? fin_len_c(P, (uint32_t)r) : 0u;
+            write_keys(P, r, L, t, o + keys_before<EXPAND_GROUP>((uint32_t)(r >> 32), L, un, lane));
         }
-        while (many) {
-            const uint32_t j = __ffs(many) - 1;
-            many &= many - 1;
-            const uint64_t t = t0 + j;
-            const uint32_t m = __shfl_sync(0xFFFFFFFFu, ml, j);
-            uint64_t o = __shfl_sync(0xFFFFFFFFu, ol, j);
-            for (uint32_t i0 = 0; i0 < m; i0 += 32) {
-                const uint32_t i = i0 + lane;
-                uint64_t r = 0;
-                uint32_t L = 0;
-                if (i < m) {
-                    r = P.recs[t * P.unit_cap + i];
-                    L = fin_len_c(P, (uint32_t)r);
-                }
-                const uint32_t before = keys_before<32>((uint32_t)(r >> 32), L, un, lane);
-                write_keys(P, r, L, t, o + before);
-                // (unordered units end after one round)
-                o += __shfl_sync(0xFFFFFFFFu, before + L, 31);
+        // larger units: their rounds of 32 records, each loaded a round ahead
+        uint32_t mn = 0, in = 0;
+        auto next_many = [&](bool fresh) {
+            if (fresh) {
+                jn = __ffs(many) - 1;
+                many &= many - 1;
+                mn = __shfl_sync(0xFFFFFFFFu, ml, jn);
+                in = 0;
             }
+            rn = in + lane < mn ? P.recs[(t0 + jn) * P.unit_cap + in + lane] : 0ull;
+            in += 32;
+        };
+        more = many != 0;
+        if (more) next_many(true);
+        uint64_t o = 0;
+        while (more) {
+            const uint64_t r = rn, t = t0 + jn;
+            // the unit's first round starts at its offset
+            const uint64_t ob = __shfl_sync(0xFFFFFFFFu, ol, jn);
+            if (in == 32) o = ob;
+            const bool fresh = in >= mn;
+            more = !fresh || many != 0;
+            if (more) next_many(fresh);
+            const uint32_t L = (uint32_t)r ? fin_len_c(P, (uint32_t)r) : 0u;
+            const uint32_t before = keys_before<32>((uint32_t)(r >> 32), L, un, lane);
+            write_keys(P, r, L, t, o + before);
+            // (unordered units end after one round)
+            o += __shfl_sync(0xFFFFFFFFu, before + L, 31);
         }
     }
     if (threadIdx.x == 0 && c == gridDim.x - 1) {
@@ -316,20 +334,25 @@ struct Plan {
     size_t smem_emit;
     uint32_t e_tbl_words, e_tbl_m_words;
     // the window kernel takes the scan (the fields above then describe the
-    // plan that its options would otherwise run): the prefix bitmap its
-    // candidates are tested against, its words in shared memory
+    // plan that its options would otherwise run): words of the prefix bitmap
+    // in its shared memory
     bool win;
-    uint32_t wf_k, wf_words;
+    uint32_t wf_words;
     size_t smem_win;
     void *kernel_win, *kernel_win_small;
+    // the dense scan kernel takes it: its tables in shared memory
+    bool dsc;
+    uint32_t d_rep, d_c_words, d_e_words, d_m_words;
+    size_t smem_d;
+    void *kernel_d;
 };
 
 enum { SCAN_QUEUED = 1, SCAN_REGISTER = 2, SCAN_SERIAL = 3 };
 
 struct WsLayout {
     uint64_t hdr, tile_m, tile_k, key_off, chunk, ovf, recs, bounds, defer, dbatch, total;
-    uint64_t wbuf;
-    uint32_t n_tiles, n_chunks, defer_cap, dbatch_cap, wbuf_cap;
+    uint64_t wbuf, wcnt;
+    uint32_t n_tiles, n_chunks, defer_cap, dbatch_cap, wsub_cap, wsubs;
 };
 
 // entries per slice the resolver kernel's buffer holds (more go to the
@@ -345,6 +368,7 @@ static inline uint64_t al256(uint64_t x) { return (x + 255) & ~255ull; }
 
 static WsLayout ws_layout(uint64_t n_bytes, uint32_t n_seg, const Plan &pl) {
     WsLayout L{};
+    const bool entries = pl.win || pl.dsc;  // the entry buffer in place of the queues
     const uint64_t ub = 1ull << pl.unit_shift;
     const uint64_t nt = (n_bytes + ub - 1) / ub;
     L.n_tiles = (uint32_t)nt;
@@ -359,6 +383,7 @@ static WsLayout ws_layout(uint64_t n_bytes, uint32_t n_seg, const Plan &pl) {
     L.hdr = put(sizeof(WsHeader));
     // one memset zeroes the header and the counts (the record counts only
     // where they are kept apart from the key counts)
+    L.wcnt = put(entries ? (uint64_t)WSUB_MAX * WSUB_STRIDE * 4 : 0);
     L.chunk = put((uint64_t)CHUNKS_MAX * 8);
     L.tile_k = put(nt * 8);
     L.tile_m = put(nt * 4);
@@ -370,16 +395,20 @@ static WsLayout ws_layout(uint64_t n_bytes, uint32_t n_seg, const Plan &pl) {
     L.bounds = put(n_seg > 1 ? (pl.queued ? nt * 4 : nt * SEGW * 4) : 0);
     // register-staged plans: the queues handed to the resolver kernel (at
     // most one batch per slice, plus each warp's last)
-    const bool defer = pl.defer && !pl.win;
+    const bool defer = pl.defer && !entries;
     const uint64_t dcap = defer ? std::min<uint64_t>(nt * DEFER_PER_UNIT, 0xFFFFFF00ull) : 0;
     L.defer_cap = (uint32_t)dcap;
     L.dbatch_cap = defer ? (uint32_t)std::min<uint64_t>(nt + 4096, 0xFFFFFF00ull) : 0u;
     L.defer = put(dcap * 16);
     L.dbatch = put((uint64_t)L.dbatch_cap * 8);
-    // the window kernel's entries (the counter runs at most one reservation
-    // per warp past the capacity)
-    L.wbuf_cap = pl.win ? (uint32_t)std::min<uint64_t>(nt * WBUF_PER_UNIT, 0xF0000000ull) : 0u;
-    L.wbuf = put((uint64_t)L.wbuf_cap * 8);
+    // the window and dense kernels' entries, in parts that the warps share out between
+    // them: at least 512 entries each (a part's counter runs at most one
+    // reservation per warp past them)
+    L.wsubs = 1;
+    while (L.wsubs < WSUB_MAX && nt * WBUF_PER_UNIT >= 1024ull * L.wsubs) L.wsubs *= 2;
+    L.wsub_cap = entries ? (uint32_t)std::min<uint64_t>((nt * WBUF_PER_UNIT + L.wsubs - 1) / L.wsubs,
+                                                       0xF0000000ull) : 0u;
+    L.wbuf = put((uint64_t)L.wsub_cap * L.wsubs * 8);
     L.total = o;
     return L;
 }
@@ -829,33 +858,65 @@ static int make_scan_plan(const pfac_table *t, const pfac_match_opts *opts, Plan
     return PFAC_OK;
 }
 
+// The dense scan kernel for a plan with a record per position: 2-bit symbols,
+// one segment.  The counts and the prefix bitmap go to shared memory, then the
+// child masks and the entries where they fit, then copies of the bitmap.
+static bool plan_dense(const pfac_table *t, Plan *pl) {
+    const DevTable &T = t->dev;
+    const uint32_t k = pl->k;
+    if (T.bps != 2 || (T.W != 0 && T.W != 1 && T.W != 3)) return false;
+    const uint32_t fw = ((1u << (2 * k)) + 31) / 32, cw = (fw + (1u << T.c_shift[k]) - 1) >> T.c_shift[k];
+    auto al4 = [](uint32_t x) { return (x + 3) & ~3u; };
+    auto size = [&](uint32_t rep, uint32_t m, uint32_t e) {
+        return ((size_t)(fw << rep) + al4(cw) + al4(m) + al4(e)) * 4 + DNW * sizeof(DWarpArea);
+    };
+    if (fw % 4 || size(0, 0, 0) > SMEM_LIMIT) return false;
+    const uint32_t m = T.M[k] && size(0, T.m_words[k], 0) <= SMEM_LIMIT ? T.m_words[k] : 0u;
+    const uint32_t e = size(0, m, T.n_e[k]) <= SMEM_LIMIT ? T.n_e[k] : 0u;
+    uint32_t rep = 0;
+    while (rep < 4 && size(rep + 1, m, e) <= SMEM_LIMIT) rep++;
+    pl->kernel_d = scan_kernel_d(e != 0);
+    pl->kernel_res = dresolve_kernel((int)T.W);
+    if (!pl->kernel_d || !pl->kernel_res) return false;
+    pl->d_rep = rep;
+    pl->d_c_words = cw;
+    pl->d_m_words = m;
+    pl->d_e_words = e;
+    pl->smem_d = size(rep, m, e);
+    return true;
+}
+
 // The plan of a call: the scan plan its options ask for and, when they leave
-// every choice to the library and the table has no tuned one, the window
-// kernel over the table's filter in place of that scan.  The emit pass, which
+// every choice to the library and the table has no tuned one, in place of that
+// scan the window kernel over the table's filter, or for one segment of
+// 2-bit symbols with many matches the dense scan kernel.  The emit pass, which
 // re-scans slices with more matches than their records, stays the plan's own.
-static int make_plan(const pfac_table *t, const pfac_match_opts *opts, Plan *pl) {
+static int make_plan(const pfac_table *t, uint32_t n_seg, const pfac_match_opts *opts, Plan *pl) {
     const int rc = make_scan_plan(t, opts, pl);
     if (rc != PFAC_OK) return rc;
     const DevTable &T = t->dev;
-    if (!T.H || T.dag || pl->kind == SCAN_SERIAL || pl->unit_cap != (uint32_t)SCAP) return PFAC_OK;
+    if (T.dag || pl->kind == SCAN_SERIAL) return PFAC_OK;
     if (opts && (opts->variant || opts->prefix_depth || opts->ctas_per_sm || opts->bitmap_copies ||
                  opts->child_masks || opts->gram_filter || opts->prefix_bytes ||
                  opts->warps_per_cta || opts->scan_kernel || opts->test_wait_limit_us ||
                  opts->test_withhold_slice || opts->records_per_slice || opts->resolver))
         return PFAC_OK;
     if (t->tuned_variant || t->tuned_k || t->tuned_nw || t->tuned_kernel) return PFAC_OK;
-    // shared memory: the filter's copies, the warps' queues, then the deepest
-    // prefix bitmap held that still fits (none: candidates are tested through L2)
+    if (pl->unit_cap == (uint32_t)SLICE) {
+        void *res = pl->kernel_res;
+        pl->dsc = n_seg <= 1 && plan_dense(t, pl);
+        if (!pl->dsc) pl->kernel_res = res;
+        return PFAC_OK;
+    }
+    if (!T.H || pl->unit_cap != (uint32_t)SCAP) return PFAC_OK;
+    // shared memory: the filter's copies, the warps' queues, and the prefix
+    // bitmap the candidates are tested against, where it fits beside them
+    // (else they are tested through L2: a shallower bitmap that fits lets too
+    // many of them through, which cost more in the resolver)
     const size_t fixed = ((size_t)T.w_words << T.w_rep) * 4 + WNW * WQCAP * 4;
     if (fixed > SMEM_LIMIT) return PFAC_OK;
-    pl->wf_k = pl->k;
-    for (uint32_t k = t->kmin; k <= pl->k; k++) {
-        const uint64_t fw = ((1ull << (k * T.bps)) + 31) / 32;
-        if (fw % 4 == 0 && fixed + fw * 4 <= SMEM_LIMIT) {
-            pl->wf_k = k;
-            pl->wf_words = (uint32_t)fw;
-        }
-    }
+    const uint64_t fw = ((1ull << (pl->k * T.bps)) + 31) / 32;
+    if (fw % 4 == 0 && fixed + fw * 4 <= SMEM_LIMIT) pl->wf_words = (uint32_t)fw;
     pl->smem_win = fixed + (size_t)pl->wf_words * 4;
     pl->kernel_win = scan_kernel_w(T, T.w_rep ? WT_COPIES : WT_ONE);
     pl->kernel_win_small = scan_kernel_w(T, WT_L2);
@@ -939,9 +1000,16 @@ extern "C" int pfac_workspace_bytes(const pfac_table *t, uint64_t n_bytes, uint3
         return set_error(PFAC_EINVAL, "pfac_workspace_bytes: input longer than 2^%d bytes",
                          64 - PFAC_ID_BITS);
     Plan pl;
-    const int rc = make_plan(t, opts, &pl);
+    const int rc = make_plan(t, n_segments, opts, &pl);
     if (rc) return rc;
     *bytes = ws_layout(n_bytes, n_segments, pl).total;
+    if (pl.unit_cap == (uint32_t)SLICE && n_segments > 1) {
+        // enough for fewer segments too (a chunk of a longer text), where
+        // another kernel may take the call
+        Plan one;
+        if (make_plan(t, 1, opts, &one) == PFAC_OK)
+            *bytes = std::max(*bytes, ws_layout(n_bytes, 1, one).total);
+    }
     return PFAC_OK;
 }
 
@@ -950,7 +1018,7 @@ extern "C" int pfac_match_plan(const pfac_table *t, const pfac_match_opts *opts,
     clear_error();
     if (!t || !out) return set_error(PFAC_EINVAL, "pfac_match_plan: NULL argument");
     Plan pl;
-    const int rc = make_plan(t, opts, &pl);
+    const int rc = make_plan(t, 1, opts, &pl);
     if (rc) return rc;
     memset(out, 0, sizeof *out);
     out->smem_bytes = (uint32_t)pl.smem;
@@ -1001,7 +1069,7 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
         return set_error(PFAC_EINVAL, "pfac_match: position_base + n_bytes reaches 2^%d",
                          64 - PFAC_ID_BITS);
     Plan pl;
-    int rc = make_plan(t, opts, &pl);
+    int rc = make_plan(t, n_segments, opts, &pl);
     if (rc) return rc;
     const WsLayout L = ws_layout(n_bytes, n_segments, pl);
     if (workspace_bytes < L.total)
@@ -1009,7 +1077,9 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
                          (unsigned long long)workspace_bytes, (unsigned long long)L.total);
     const bool reg = pl.kind == SCAN_REGISTER;
     const size_t smem_emit = reg ? pl.smem_emit : pl.smem;
-    rc = pl.win ? prepare_kernel(pl.kernel_win, pl.smem_win) : prepare_kernel(pl.kernel, pl.smem);
+    rc = pl.win   ? prepare_kernel(pl.kernel_win, pl.smem_win)
+         : pl.dsc ? prepare_kernel(pl.kernel_d, pl.smem_d)
+                  : prepare_kernel(pl.kernel, pl.smem);
     if (!rc && pl.kernel_emit != pl.kernel) rc = prepare_kernel(pl.kernel_emit, smem_emit);
     if (rc) return rc;
 
@@ -1066,22 +1136,24 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
     P.wait_limit_ns = opts && opts->test_wait_limit_us ? (uint64_t)opts->test_wait_limit_us * 1000
                                                        : WAIT_LIMIT_NS;
     P.withhold_unit = opts && opts->test_withhold_slice ? opts->test_withhold_slice - 1 : UNIT_NONE;
+    if (pl.win || pl.dsc) {
+        P.wbuf = (uint64_t *)(W + L.wbuf);
+        P.wcnt = (uint32_t *)(W + L.wcnt);
+        P.wsub_cap = L.wsub_cap;
+        P.wsub_mask = L.wsubs - 1;
+    }
     if (pl.win) {
         const DevTable &T = t->dev;
         const uint32_t bits = T.w_packed ? 2 * T.w_gw : 8 * T.w_gw;
-        P.wbuf = (uint64_t *)(W + L.wbuf);
-        P.wbuf_cap = L.wbuf_cap;
         P.w_words = T.w_words;
         P.w_rep = T.w_rep;
         P.w_gm = gram_mul(bits);
         P.w_glen = T.w_glen;
         P.w_badmask = T.w_short ? 0x01010101u * ((0xFFu << T.bps) & 0xFFu) : 0u;
-        P.wf = T.F[pl.wf_k];
         P.wf_words = pl.wf_words;
-        P.wf_k = pl.wf_k;
         P.unordered = 1;
         P.chunk_adds = P.chunk_shift == CHUNK_SHIFT_MIN;
-    } else if (pl.defer) {
+    } else if (pl.defer && !pl.dsc) {
         P.defer = (uint4 *)(W + L.defer);
         P.defer_cap = L.defer_cap;
         P.dbatch = (uint2 *)(W + L.dbatch);
@@ -1118,13 +1190,24 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
         e = cudaLaunchKernel(small ? pl.kernel_win_small : pl.kernel_win,
                              dim3(small || need < (uint32_t)nsm ? need : (uint32_t)nsm), dim3(nw * 32),
                              args, small ? (size_t)WNW_SMALL * WQCAP * 4 : pl.smem_win, st);
+    } else if (e == cudaSuccess && P.n_tiles && pl.dsc) {
+        MatchParams PD = P;
+        PD.rep_log2 = pl.d_rep;
+        PD.tbl_words = (((1u << (2 * pl.k)) + 31) / 32) << pl.d_rep;
+        PD.tbl_c_words = pl.d_c_words;
+        PD.tbl_m_words = pl.d_m_words;
+        PD.tbl_e_words = pl.d_e_words;
+        const uint32_t need = ((P.n_tiles + 1) / 2 + DNW - 1) / DNW;
+        void *args[] = {&PD};
+        e = cudaLaunchKernel(pl.kernel_d, dim3(need < (uint32_t)nsm ? need : (uint32_t)nsm), dim3(DNW * 32),
+                             args, pl.smem_d, st);
     } else if (e == cudaSuccess && P.n_tiles) {
         int emit = 0;
         void *args[] = {&P, &emit};
         e = cudaLaunchKernel(pl.kernel, dim3(grid), dim3(nthreads), args, pl.smem, st);
     }
-    if (e == cudaSuccess && P.n_tiles && (pl.win || pl.defer)) {
-        // the handed-over queues (or the window kernel's entries): prefix bitmap, counts and entries through
+    if (e == cudaSuccess && P.n_tiles && (pl.win || pl.dsc || pl.defer)) {
+        // the handed-over queues (or the window or dense kernel's entries): prefix bitmap, counts and entries through
         // L2 (one bitmap copy)
         MatchParams P3 = P;
         P3.rep_log2 = 0;
@@ -1140,8 +1223,8 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-        // four units per warp where that is all there are (chunks of 32)
-        const uint32_t span = P.chunk_shift == CHUNK_SHIFT_MIN ? 4u : 32u;
+        // a chunk's units over its CTA's eight warps, 32 at most at a time
+        const uint32_t span = P.chunk_shift < 8 ? (1u << P.chunk_shift) / 8 : 32u;
         k_expand<<<n_chunks ? n_chunks : 1, 256, 0, st>>>(P, span);
         e = cudaGetLastError();
     }

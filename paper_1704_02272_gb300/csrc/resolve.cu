@@ -16,11 +16,21 @@ void *resolve_kernel(int w) {
 
 void *wresolve_kernel(int w) {
     switch (w) {
-        case 0: return (void *)k_wresolve<0>;
-        case 1: return (void *)k_wresolve<1>;
-        case 2: return (void *)k_wresolve<2>;
-        case 3: return (void *)k_wresolve<3>;
-        case 8: return (void *)k_wresolve<8>;
+        case 0: return (void *)k_wresolve<0, 0>;
+        case 1: return (void *)k_wresolve<1, 0>;
+        case 2: return (void *)k_wresolve<2, 0>;
+        case 3: return (void *)k_wresolve<3, 0>;
+        case 8: return (void *)k_wresolve<8, 0>;
+        default: return nullptr;
+    }
+}
+
+// pending records of the dense scan kernel (2-bit symbols)
+void *dresolve_kernel(int w) {
+    switch (w) {
+        case 0: return (void *)k_wresolve<0, 1>;
+        case 1: return (void *)k_wresolve<1, 1>;
+        case 3: return (void *)k_wresolve<3, 1>;
         default: return nullptr;
     }
 }
