@@ -323,7 +323,7 @@ int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uint64_t n_byt
 
 /*
  * pfac_match - synchronous form of pfac_match_async: allocates the workspace
- * with the stream-ordered allocator, matches, waits for the stream and writes
+ * with the stream-ordered allocator (a pool of the library's own), matches, waits for the stream and writes
  * the total match count to the host *n_out.  Returns PFAC_ENOSPC when
  * count > out_capacity (the first out_capacity keys are valid and *n_out holds
  * the full count, so a second call with a larger buffer succeeds).
@@ -389,7 +389,9 @@ int pfac_verify(const pfac_table *t, const uint8_t *d_input, uint64_t n_bytes,
                 uint64_t n_keys, uint64_t *d_out, uint64_t *d_count, void *cuda_stream);
 
 /* pfac_match_host_release - free the buffers pfac_match_host keeps for the
- * current device (waits for the device first).  Library extension. */
+ * current device (waits for the device first), and give back what the scratch
+ * pool of pfac_match and pfac_verify keeps between calls (at most 64 MiB per
+ * device).  Library extension. */
 void pfac_match_host_release(void);
 
 /*

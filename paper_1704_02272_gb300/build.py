@@ -31,7 +31,7 @@ def nvcc() -> str:
 
 
 def sources():
-    srcs = ["builder.cpp", "tune.cpp", "serve.cpp", "host.cpp", "window.cpp", "match.cu", "noalloc.cu",
+    srcs = ["builder.cpp", "tune.cpp", "serve.cpp", "host.cpp", "window.cpp", "pool.cpp", "match.cu", "noalloc.cu",
             "verify.cu", "resolve.cu", "scan_dense.cu", "scan_d.cu", "table_io.cpp"] + [f"scan_bps{i}.cu" for i in range(1, 9)] + \
         [f"scan_r{b}_{g}.cu" for b in (8, 2) for g in ("g0_f", "g0_fe", "g1_f", "g1_fe", "d0", "d1")] + \
         [f"scan_w{s}.cu" for s in (1, 2, 4, 8, 16)]

@@ -109,6 +109,7 @@ cudaError_t ctx_prepare(HostCtx &c, uint64_t in_b, uint64_t seg_b, uint64_t ws_b
 }  // namespace
 
 extern "C" void pfac_match_host_release(void) {
+    scratch_trim();
     std::lock_guard<std::mutex> lk(g_host_mu);
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEV) return;

@@ -1,6 +1,7 @@
 // Host-side table object and error reporting shared by the library's
 // translation units.
 #pragma once
+#include <cuda_runtime.h>
 #include <stdarg.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -44,5 +45,13 @@ void clear_error();
 // (with a message naming `who`), so that no kernel is launched on one GPU
 // with another GPU's pointers.
 int check_table_device(const pfac_table *t, void *cuda_stream, const char *who);
+
+// Stream-ordered scratch from the library's own pool of the current device
+// (freed with cudaFreeAsync), and giving back what the pool keeps.
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st);
+void scratch_trim();
+
+// The current CUDA context (nullptr when it cannot be told).
+void *current_context();
 
 }  // namespace pfac

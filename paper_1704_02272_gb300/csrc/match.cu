@@ -1274,31 +1274,29 @@ extern "C" int pfac_match(const pfac_table *t, const uint8_t *d_input, uint64_t 
     uint64_t ws_bytes = 0;
     int rc0 = pfac_workspace_bytes(t, n_bytes, n_segments, opts, &ws_bytes);
     if (rc0) return rc0;
-    void *ws = nullptr, *small = nullptr;
-    cudaError_t e = cudaMallocAsync(&ws, ws_bytes, st);
-    if (e == cudaSuccess) e = cudaMallocAsync(&small, 256, st);
+    // the workspace, then the count and the status, read back in one copy
+    void *ws = nullptr;
+    cudaError_t e = scratch_alloc(&ws, ws_bytes + 256, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        if (ws) cudaFreeAsync(ws, st);
         return set_error(e == cudaErrorMemoryAllocation ? PFAC_ENOMEM : PFAC_ECUDA,
                          "pfac_match: workspace allocation: %s", cudaGetErrorString(e));
     }
-    uint64_t *d_cnt = (uint64_t *)small;
-    int32_t *d_st = (int32_t *)((uint8_t *)small + 128);
+    uint64_t *d_cnt = (uint64_t *)((uint8_t *)ws + ws_bytes);
+    int32_t *d_st = (int32_t *)(d_cnt + 1);
     int rc = pfac_match_async(t, d_input, n_bytes, d_seg_offsets, n_segments, d_out_keys,
                               out_capacity, d_cnt, d_st, ws, ws_bytes, opts, cuda_stream);
     struct {
         uint64_t cnt;
         int32_t st;
-    } h{0, 0};
+        int32_t pad;
+    } h{0, 0, 0};
     if (rc == PFAC_OK) {
-        e = cudaMemcpyAsync(&h.cnt, d_cnt, 8, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&h.st, d_st, 4, cudaMemcpyDeviceToHost, st);
+        e = cudaMemcpyAsync(&h, d_cnt, sizeof h, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) rc = set_error(PFAC_ECUDA, "pfac_match: %s", cudaGetErrorString(e));
     }
     cudaFreeAsync(ws, st);
-    cudaFreeAsync(small, st);
     if (rc) return rc;
     *n_out = h.cnt;
     if (h.st != PFAC_OK)

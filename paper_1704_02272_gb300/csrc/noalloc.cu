@@ -52,12 +52,18 @@ CtxGetCurrentFn ctx_get_current() {
     return fn;
 }
 
-void *current_context() {
+}  // namespace
+
+void *pfac::current_context() {
     void *ctx = nullptr;
     CtxGetCurrentFn f = ctx_get_current();
     if (!f || f(&ctx) != 0) return nullptr;
     return ctx;
 }
+
+namespace {
+
+using pfac::current_context;
 
 // Device address of this device's copy of the array.  In host code the
 // array's name is only a host-side stand-in, so the address must come from

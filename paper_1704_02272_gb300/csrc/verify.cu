@@ -167,7 +167,7 @@ extern "C" int pfac_verify(const pfac_table *t, const uint8_t *d_input, uint64_t
                                 : set_error(PFAC_ECUDA, "pfac_verify: %s", cudaGetErrorString(e));
     }
     void *scratch = nullptr;
-    cudaError_t e = cudaMallocAsync(&scratch, V.n_tiles * 8 + n_keys + 16, st);
+    cudaError_t e = scratch_alloc(&scratch, V.n_tiles * 8 + n_keys + 16, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return set_error(e == cudaErrorMemoryAllocation ? PFAC_ENOMEM : PFAC_ECUDA,
