@@ -277,7 +277,7 @@ int pfac_workspace_bytes(const pfac_table *t, uint64_t n_bytes, uint32_t n_segme
  * choice and its pattern set makes a window filter that pays (a filter over
  * short windows of the text, every S-th position looked up; built with the
  * table), the scan pass runs over that filter; the fields then describe the
- * plan that runs without it and whose emit pass the call uses.
+ * plan that runs without it.
  */
 typedef struct {
     uint32_t variant;        /* 1 or 2, as pfac_match_opts.variant */

@@ -89,6 +89,8 @@ __global__ void __launch_bounds__(DNW * 32, 1) k_scand(const __grid_constant__ M
         for (uint32_t i = threadIdx.x; i < P.tbl_e_words; i += DNW * 32) Es[i] = __ldg(P.E + i);
     }
     __syncthreads();
+    // from here on the call's counters are used, zeroed by the kernel before
+    dep_wait();
     if (gw >= n_pairs) return;
 
     const uint64_t N = P.n, N16 = N & ~15ull;

@@ -1108,6 +1108,7 @@ __global__ void __launch_bounds__(NW * 32, 1) k_scanq(const __grid_constant__ Ma
     constexpr bool emit = EMIT != 0;
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (emit) dep_wait();
     const uint32_t n_units = emit ? *(volatile uint32_t *)&P.hdr->ovf_count : P.n_tiles;
     const uint32_t gw = blockIdx.x * NW + warp, gstride = gridDim.x * NW;
     if (blockIdx.x * NW >= n_units) {  // the whole CTA has no unit

@@ -142,8 +142,8 @@ __device__ __forceinline__ uint32_t w_filter(const uint32_t (&w)[9], const WCons
 
 // One match: a record in the slice's space while it has room (in any order),
 // and the slice's counts: records above bit UNIT_KEY_BITS of its word, keys
-// below, so that one atomic takes the slot and counts the keys.  The first
-// match past the space lists the slice for the emit pass.  With few slices
+// below, so that one atomic takes the slot and counts the keys.  (A slice with
+// more matches than its space is walked again by the expansion.)  With few slices
 // the chunks' key counts are added up here too; with many, neighbouring
 // matches would queue on one chunk's word (1 GiB of packets: 0.8 instead of
 // 0.36 ms), and k_reduce sums them.
@@ -154,7 +154,6 @@ __device__ __forceinline__ void w_emit(const MatchParams &P, uint32_t u, uint32_
     const uint32_t rank = (uint32_t)(atomicAdd((unsigned long long *)(P.tile_k + u),
                                                (1ull << UNIT_KEY_BITS) | keys) >> UNIT_KEY_BITS);
     if (rank < cap) P.recs[(size_t)u * cap + rank] = ((uint64_t)pos << 32) | fin;
-    else if (rank == cap) P.ovf_list[chk(P, atomicAdd(&P.hdr->ovf_count, 1u), P.n_tiles)] = u;
     if (P.chunk_adds) atomicAdd((unsigned long long *)(P.chunk + (u >> P.chunk_shift)), keys);
 }
 
@@ -382,8 +381,6 @@ __global__ void __launch_bounds__((TB == WT_L2 ? WNW_SMALL : WNW) * 32, 1)
     const uint32_t gw = blockIdx.x * NW + warp, gstride = gridDim.x * NW;
     if (blockIdx.x * NW >= n_pairs) return;
 
-    if (P.n_seg > 1) unit_segments(P, gw, gstride, lane);
-
     // shared memory: H (all copies), the prefix bitmap, the queues
     const uint32_t hwords = TB == WT_L2 ? 0u : P.w_words << P.w_rep;
     uint32_t *Fs = reinterpret_cast<uint32_t *>(smem) + hwords;
@@ -394,6 +391,9 @@ __global__ void __launch_bounds__((TB == WT_L2 ? WNW_SMALL : WNW) * 32, 1)
         w_fill<NW * 32>(Fs, P.F, P.wf_words, 0u, blockIdx.x * 32u);
         __syncthreads();
     }
+    // from here on the call's counters are used, zeroed by the kernel before
+    dep_wait();
+    if (P.n_seg > 1) unit_segments(P, gw, gstride, lane);
     WConst K;
     K.gm = P.w_gm;
     K.tbl = P.T.H;
@@ -544,6 +544,7 @@ __global__ void __launch_bounds__(RES_WARPS * 32, RES_CTAS)
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     WTail &T = tails[warp];
+    dep_wait();
     const uint32_t gw = blockIdx.x * RES_WARPS + warp, gs = gridDim.x * RES_WARPS;
     // the buffer's parts: lane l counts those of parts l and l + 32
     const uint32_t parts = P.wsub_mask + 1;

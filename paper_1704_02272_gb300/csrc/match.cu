@@ -159,10 +159,18 @@ __device__ __forceinline__ uint64_t block_excl_scan(uint64_t v, uint64_t *sh, ui
     return r;
 }
 
+// Zeroes the head of the workspace (n 16-byte words): a kernel rather than a
+// memset, so that the scan's table fill overlaps it.
+__global__ void __launch_bounds__(256) k_zero(uint4 *p, uint64_t n) {
+    for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256)
+        p[i] = make_uint4(0, 0, 0, 0);
+}
+
 // Key counts of the chunks of units, where they are not added up as matches
 // are found.
 __global__ void __launch_bounds__(256) k_reduce(const MatchParams P) {
     __shared__ uint64_t sh[33];
+    dep_wait();
     const uint64_t t0 = (uint64_t)blockIdx.x << P.chunk_shift;
     uint64_t sum = 0;
     for (uint64_t i = threadIdx.x; i < (1ull << P.chunk_shift); i += 256)
@@ -219,18 +227,38 @@ __device__ __forceinline__ void write_keys(const MatchParams &P, uint64_t r, uin
         if (o < P.cap) P.out[o] = pk | __ldg(ids + e);
 }
 
-__global__ void __launch_bounds__(256) k_expand(const MatchParams P, const uint32_t span) {
+// The keys of a unit whose records were not kept, where no emit pass follows:
+// a warp walks its starts from the root, 32 at a time, in position order.
+static __device__ __noinline__ void expand_unit(const MatchParams *PP, uint64_t t, uint64_t o, uint32_t lane) {
+    const MatchParams &P = *PP;
+    const uint64_t us = t << SLICE_SHIFT;
+    for (uint32_t p0 = 0; p0 < (uint32_t)SLICE; p0 += 32) {
+        const uint32_t pos = p0 + lane;
+        uint32_t fin = 0, L = 0;
+        if (us + pos < P.starts_end) {
+            fin = w_walk_any(P, us, pos, w_limit(P, (uint32_t)t, us + pos));
+            if (fin) L = fin_len_c(P, fin);
+        }
+        const uint32_t before = keys_before<32>(pos, L, false, lane);
+        write_keys(P, ((uint64_t)pos << 32) | fin, L, t, o + before);
+        o += __shfl_sync(0xFFFFFFFFu, before + L, 31);
+    }
+}
+
+__global__ void __launch_bounds__(256, 8) k_expand(const __grid_constant__ MatchParams P, const uint32_t span) {
     __shared__ uint64_t sh[33];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t grp = lane / EXPAND_GROUP, gl = lane % EXPAND_GROUP;
     const bool un = P.unordered != 0;
     const uint32_t c = blockIdx.x;
+    dep_wait();
     uint64_t base = 0;
     {
         uint64_t v = 0;
         for (uint32_t i = threadIdx.x; i < c; i += 256) v += __ldcg(P.chunk + i);
         block_excl_scan(v, sh, base);
     }
+    bool over = false;
     const uint64_t c_end = ((uint64_t)c + 1) << P.chunk_shift;
     const uint64_t t_end = c_end < P.n_tiles ? c_end : P.n_tiles;
     for (uint64_t b0 = (uint64_t)c << P.chunk_shift; b0 < t_end; b0 += 8 * span) {
@@ -242,6 +270,7 @@ __global__ void __launch_bounds__(256) k_expand(const MatchParams P, const uint3
         const uint64_t ol = block_excl_scan(kl & ((1ull << UNIT_KEY_BITS) - 1), sh, tot) + base;
         base += tot;
         if (ml > P.unit_cap) P.key_off[tl] = ol;
+        over |= ml > P.unit_cap;
         uint32_t few = __ballot_sync(0xFFFFFFFFu, ml != 0 && ml <= EXPAND_GROUP);
         uint32_t many = __ballot_sync(0xFFFFFFFFu, ml > EXPAND_GROUP && ml <= P.unit_cap);
         // the records of the next four units are loaded while the keys of
@@ -305,8 +334,26 @@ __global__ void __launch_bounds__(256) k_expand(const MatchParams P, const uint3
                                          : (P.n == 0 && P.seg[0] == 0);
             if (!ok) atomicOr(&P.hdr->status, ST_BADSEG);
         }
-        // no unit, no emit pass: the status is published here
-        if (P.n_tiles == 0) publish_status(P, 1);
+    }
+    // where no emit pass follows, this kernel re-walks the units whose records
+    // were not kept and publishes the status: its last chunk's CTA can, as no
+    // other one changes it (in the checked build every one may)
+    if (P.no_emit && __any_sync(0xFFFFFFFFu, over)) {
+        __syncwarp();
+        for (uint64_t b0 = (uint64_t)c << P.chunk_shift; b0 < t_end; b0 += 8 * span) {
+            const uint64_t t0 = b0 + warp * span, tl = t0 + lane;
+            const bool full = lane < span && tl < t_end && (P.tile_k[tl] >> UNIT_KEY_BITS) > P.unit_cap;
+            uint32_t m = __ballot_sync(0xFFFFFFFFu, full && un);
+            while (m) {
+                const uint32_t j = __ffs(m) - 1;
+                m &= m - 1;
+                expand_unit(&P, t0 + j, P.key_off[t0 + j], lane);
+            }
+        }
+    }
+    if (P.no_emit || P.n_tiles == 0) {
+        if (CHECKED) __syncthreads();
+        if (threadIdx.x == 0 && (CHECKED || c == gridDim.x - 1)) publish_status(P, CHECKED ? gridDim.x : 1);
     }
 }
 
@@ -889,8 +936,7 @@ static bool plan_dense(const pfac_table *t, Plan *pl) {
 // The plan of a call: the scan plan its options ask for and, when they leave
 // every choice to the library and the table has no tuned one, in place of that
 // scan the window kernel over the table's filter, or for one segment of
-// 2-bit symbols with many matches the dense scan kernel.  The emit pass, which
-// re-scans slices with more matches than their records, stays the plan's own.
+// 2-bit symbols with many matches the dense scan kernel.
 static int make_plan(const pfac_table *t, uint32_t n_seg, const pfac_match_opts *opts, Plan *pl) {
     const int rc = make_scan_plan(t, opts, pl);
     if (rc != PFAC_OK) return rc;
@@ -980,6 +1026,25 @@ int check_table_device(const pfac_table *t, void *cuda_stream, const char *who) 
                              "lives on device %d", who, sd, t->device);
     }
     return PFAC_OK;
+}
+
+// Launches a kernel that may start while the one before it still runs
+// (dep_wait in kernels.cuh); with dep == false an ordinary launch.
+static cudaError_t launch(const void *fn, uint32_t grid, uint32_t block, void **args, size_t smem,
+                          cudaStream_t st, bool dep) {
+    cudaLaunchConfig_t c;
+    memset(&c, 0, sizeof c);
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute a;
+    memset(&a, 0, sizeof a);
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &a;
+    c.numAttrs = dep ? 1 : 0;
+    return cudaLaunchKernelExC(&c, fn, args);
 }
 
 static int sm_count() {
@@ -1080,7 +1145,7 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
     rc = pl.win   ? prepare_kernel(pl.kernel_win, pl.smem_win)
          : pl.dsc ? prepare_kernel(pl.kernel_d, pl.smem_d)
                   : prepare_kernel(pl.kernel, pl.smem);
-    if (!rc && pl.kernel_emit != pl.kernel) rc = prepare_kernel(pl.kernel_emit, smem_emit);
+    if (!rc && !pl.win && !pl.dsc && pl.kernel_emit != pl.kernel) rc = prepare_kernel(pl.kernel_emit, smem_emit);
     if (rc) return rc;
 
     cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -1137,6 +1202,9 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
                                                        : WAIT_LIMIT_NS;
     P.withhold_unit = opts && opts->test_withhold_slice ? opts->test_withhold_slice - 1 : UNIT_NONE;
     if (pl.win || pl.dsc) {
+        // the window kernel's re-walks of full slices are the expansion's (the
+        // dense kernel has a record for every position)
+        P.no_emit = 1;
         P.wbuf = (uint64_t *)(W + L.wbuf);
         P.wcnt = (uint32_t *)(W + L.wcnt);
         P.wsub_cap = L.wsub_cap;
@@ -1166,9 +1234,20 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
 
     // header, and for the slice kernels the per-unit record and key counts
     // (the scan pass writes them only for units with kept survivors)
-    cudaError_t e = cudaMemsetAsync(P.hdr, 0,
-                                    pl.win ? L.tile_m : (pl.queued ? L.key_off : sizeof(WsHeader)), st);
+    const bool ent = pl.win || pl.dsc;
+    const uint64_t zero = pl.win ? L.tile_m : (pl.queued ? L.key_off : sizeof(WsHeader));
     const int nsm = sm_count();
+    cudaError_t e;
+    if (ent) {
+        uint4 *zp = (uint4 *)P.hdr;
+        uint64_t zn = zero / 16;
+        void *args[] = {&zp, &zn};
+        const uint64_t zb = (zn + 1023) / 1024;
+        e = launch((const void *)k_zero, (uint32_t)std::min<uint64_t>(zb ? zb : 1, (uint64_t)nsm * 4), 256, args,
+                   0, st, false);
+    } else {
+        e = cudaMemsetAsync(P.hdr, 0, zero, st);
+    }
     const uint32_t cps = opts && opts->ctas_per_sm ? opts->ctas_per_sm : 1;
     if (e == cudaSuccess && n_segments > 1 && P.n_tiles && !pl.win) {
         if (pl.queued) k_unitseg<<<nsm * 4, 256, 0, st>>>(P);
@@ -1187,9 +1266,9 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
         const uint32_t nw = small ? WNW_SMALL : WNW;
         const uint32_t need = (n_pairs + nw - 1) / nw;
         void *args[] = {&P};
-        e = cudaLaunchKernel(small ? pl.kernel_win_small : pl.kernel_win,
-                             dim3(small || need < (uint32_t)nsm ? need : (uint32_t)nsm), dim3(nw * 32),
-                             args, small ? (size_t)WNW_SMALL * WQCAP * 4 : pl.smem_win, st);
+        e = launch(small ? pl.kernel_win_small : pl.kernel_win,
+                   small || need < (uint32_t)nsm ? need : (uint32_t)nsm, nw * 32, args,
+                   small ? (size_t)WNW_SMALL * WQCAP * 4 : pl.smem_win, st, true);
     } else if (e == cudaSuccess && P.n_tiles && pl.dsc) {
         MatchParams PD = P;
         PD.rep_log2 = pl.d_rep;
@@ -1199,8 +1278,7 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
         PD.tbl_e_words = pl.d_e_words;
         const uint32_t need = ((P.n_tiles + 1) / 2 + DNW - 1) / DNW;
         void *args[] = {&PD};
-        e = cudaLaunchKernel(pl.kernel_d, dim3(need < (uint32_t)nsm ? need : (uint32_t)nsm), dim3(DNW * 32),
-                             args, pl.smem_d, st);
+        e = launch(pl.kernel_d, need < (uint32_t)nsm ? need : (uint32_t)nsm, DNW * 32, args, pl.smem_d, st, true);
     } else if (e == cudaSuccess && P.n_tiles) {
         int emit = 0;
         void *args[] = {&P, &emit};
@@ -1214,23 +1292,26 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
         P3.tbl_e_words = 0;
         P3.tbl_m_words = 0;
         void *args[] = {&P3};
-        e = cudaLaunchKernel(pl.kernel_res, dim3(nsm * RES_CTAS), dim3(RES_WARPS * 32), args, 0, st);
+        // (small calls: no more warps than their entry buffer has blocks)
+        const uint32_t full = (uint32_t)nsm * RES_CTAS;
+        const uint64_t blocks = ((uint64_t)P.n_tiles * WBUF_PER_UNIT + 255) / 256;
+        e = launch(pl.kernel_res, ent && blocks < full ? (uint32_t)blocks : full, RES_WARPS * 32, args, 0, st, ent);
     }
     if (e == cudaSuccess && opts && opts->ev_scan_end)
         e = cudaEventRecord((cudaEvent_t)opts->ev_scan_end, st);
     if (e == cudaSuccess && P.n_tiles && !P.chunk_adds) {
-        k_reduce<<<n_chunks, 256, 0, st>>>(P);
-        e = cudaGetLastError();
+        void *args[] = {&P};
+        e = launch((const void *)k_reduce, n_chunks, 256, args, 0, st, true);
     }
     if (e == cudaSuccess) {
         // a chunk's units over its CTA's eight warps, 32 at most at a time
         const uint32_t span = P.chunk_shift < 8 ? (1u << P.chunk_shift) / 8 : 32u;
-        k_expand<<<n_chunks ? n_chunks : 1, 256, 0, st>>>(P, span);
-        e = cudaGetLastError();
+        void *args[] = {&P, (void *)&span};
+        e = launch((const void *)k_expand, n_chunks ? n_chunks : 1, 256, args, 0, st, true);
     }
     if (e == cudaSuccess && opts && opts->ev_emit_begin)
         e = cudaEventRecord((cudaEvent_t)opts->ev_emit_begin, st);
-    if (e == cudaSuccess && P.n_tiles) {
+    if (e == cudaSuccess && P.n_tiles && !P.no_emit) {
         int emit = 1;
         if (reg) {
             // the queued kernel re-scans the overflowing slices with its own
@@ -1248,10 +1329,10 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
             const uint32_t grid_e =
                 (uint64_t)nsm * cps < want_e ? (uint32_t)nsm * cps : (uint32_t)want_e;
             void *args[] = {&P2, &emit};
-            e = cudaLaunchKernel(pl.kernel_emit, dim3(grid_e), dim3(QW * 32), args, smem_emit, st);
+            e = launch(pl.kernel_emit, grid_e, QW * 32, args, smem_emit, st, true);
         } else {
             void *args[] = {&P, &emit};
-            e = cudaLaunchKernel(pl.kernel_emit, dim3(grid), dim3(nthreads), args, pl.smem, st);
+            e = launch(pl.kernel_emit, grid, nthreads, args, pl.smem, st, pl.queued);
         }
     }
     if (e == cudaSuccess && opts && opts->ev_emit_end)
