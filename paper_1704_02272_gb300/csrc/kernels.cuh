@@ -123,14 +123,16 @@ struct MatchParams {
     uint2 *dbatch;
     // window kernel: the entry buffer (position << 24 | prefix index), the
     // filter's split of shared memory and hash, the words of the prefix bitmap
-    // in shared memory (0: its candidates are tested against it through L2)
+    // and its counts in shared memory (0: its candidates are tested against it
+    // through L2)
     uint64_t *wbuf;
     uint32_t *wcnt;       // entries of each part of the buffer, WSUB_STRIDE words apart
     uint32_t wsub_cap;    // entries a part holds
     uint32_t wsub_mask;   // parts - 1 (a power of two, at most WSUB_MAX parts)
     uint32_t w_words, w_rep, w_gm, w_glen;
     uint32_t w_badmask;   // byte bits outside the symbol range, where they matter to the filter
-    uint32_t wf_words;
+    uint32_t wf_words, wc_words;
+    uint32_t w_ranked;    // entries hold the prefix index's rank
     uint32_t unordered;  // a unit's records are in no order (the expansion sorts them)
     uint32_t no_emit;    // no emit pass: the expansion re-walks units without records
 };

@@ -87,6 +87,16 @@ __device__ __forceinline__ uint32_t ld_stream4_if(bool on, const uint8_t *p) {
     return v;
 }
 
+__device__ __forceinline__ uint2 ld_stream8_if(bool on, const uint8_t *p) {
+    uint2 v = make_uint2(0, 0);
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t"
+        "@q ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];\n\t}"
+        : "+r"(v.x), "+r"(v.y)
+        : "l"(p), "r"((uint32_t)on));
+    return v;
+}
+
 __device__ __forceinline__ uint4 ld_stream16_if(bool on, const uint8_t *p) {
     uint4 v = make_uint4(0, 0, 0, 0);
     asm volatile(

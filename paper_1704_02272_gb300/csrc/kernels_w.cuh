@@ -215,9 +215,10 @@ static __device__ __noinline__ void w_walk(const MatchParams *PP, uint64_t p) {
 }
 
 // The text around a start, loaded without branches so that several starts'
-// loads overlap: two 16-byte chunks (2-bit symbols) or three words (raw
-// bytes) from the aligned address at or below p; zeros where they would pass
-// the input's end (ok false).
+// loads overlap: the aligned 16-byte (2-bit symbols) or 8-byte piece that
+// holds it, and the next one where its k symbols reach into that (every
+// scattered load costs its lane a cycle of the SM's L1); zeros where they
+// would pass the input's end (ok false).
 template <int PACKED>
 struct WText {
     uint4 a, b;
@@ -226,19 +227,28 @@ struct WText {
 
 template <int PACKED>
 __device__ __forceinline__ WText<PACKED> w_text(const MatchParams &P, bool on, uint64_t p) {
+    constexpr uint32_t PIECE = PACKED ? 16 : 8;
     WText<PACKED> t;
-    const uint64_t c = p & (PACKED ? ~15ull : ~3ull);
-    t.ok = on && c + (PACKED ? 32 : 12) <= P.n;
+    const uint64_t c = p & ~(uint64_t)(PIECE - 1);
+    t.ok = on && c + 2 * PIECE <= P.n;
+    const bool two = t.ok && ((uint32_t)p & (PIECE - 1)) + P.k > PIECE;
     const uint8_t *src = P.in + (t.ok ? c : 0ull);
     if (PACKED) {
         t.a = ld_stream16_if(t.ok, src);
-        t.b = ld_stream16_if(t.ok, src + 16);
+        t.b = ld_stream16_if(two, src + PIECE);
     } else {
-        t.a = make_uint4(ld_stream4_if(t.ok, src), ld_stream4_if(t.ok, src + 4),
-                         ld_stream4_if(t.ok, src + 8), 0u);
+        const uint2 a = ld_stream8_if(t.ok, src), b = ld_stream8_if(two, src + PIECE);
+        t.a = make_uint4(a.x, a.y, b.x, b.y);
         t.b = make_uint4(0u, 0u, 0u, 0u);
     }
     return t;
+}
+
+// The eight bytes from byte s (0 .. 7) of a 16-byte string.
+__device__ __forceinline__ uint2 bytes8(const uint4 &v, uint32_t s) {
+    const bool up = s >= 4;
+    const uint32_t x = up ? v.y : v.x, y = up ? v.z : v.y, z = up ? v.w : v.z, sh = 8 * (s & 3);
+    return make_uint2(__funnelshift_r(x, y, sh), __funnelshift_r(y, z, sh));
 }
 
 // Prefix index (k symbols) of the start p that t was loaded for, or WX_ROOT
@@ -253,8 +263,8 @@ __device__ __forceinline__ uint32_t w_prefix(const MatchParams &P, const WText<P
         return !t.ok || bad ? WX_ROOT : (w & ((1u << (2 * k)) - 1u));
     }
     // at most 6 symbols (k * bps <= 20, bps >= 3)
-    const uint32_t sh = 8 * ((uint32_t)p & 3u);
-    uint32_t lo = __funnelshift_r(t.a.x, t.a.y, sh), hi = __funnelshift_r(t.a.y, t.a.z, sh);
+    const uint2 w = bytes8(t.a, (uint32_t)p & 7u);
+    uint32_t lo = w.x, hi = w.y;
     uint32_t x = 0, bad = 0;
     for (uint32_t i = 0; i < k; i++) {
         const uint32_t s = lo & 0xFFu;
@@ -268,11 +278,12 @@ __device__ __forceinline__ uint32_t w_prefix(const MatchParams &P, const WText<P
 
 // Empties a warp's candidate queue (n <= WQCAP window positions): every start
 // a window stands for, one per lane, is tested against a prefix bitmap; the
-// survivors go to the entry buffer (position << 24 | prefix index), or are
-// walked here when it is full.
+// survivors go to the entry buffer (position << 24 | prefix index, or its rank
+// where the bitmap and its counts are in shared memory), or are walked here
+// when it is full.
 template <int PACKED, int S>
 __device__ __forceinline__ void w_flush(const MatchParams &P, const uint32_t *q, uint32_t n,
-                                        const uint32_t *Fs, uint32_t gw, uint32_t gstride,
+                                        const uint32_t *Fs, const uint32_t *Cs, uint32_t gw, uint32_t gstride,
                                         uint32_t lane) {
     const uint32_t lt = (1u << lane) - 1u;
     constexpr int R = PACKED ? 2 : 4;  // rounds of 32 starts whose loads overlap
@@ -298,7 +309,8 @@ __device__ __forceinline__ void w_flush(const MatchParams &P, const uint32_t *q,
             const uint32_t fx = x == WX_ROOT ? 0u : (uint32_t)chk(P, x, 1ull << (P.k * P.T.bps));
             const uint32_t fw = Fs ? Fs[fx >> 5] : __ldg(P.F + (fx >> 5));
             const bool keep = p != ~0ull && (x == WX_ROOT || ((fw >> (fx & 31)) & 1u));
-            en[r] = (p << 24) | x;
+            const uint32_t low = Fs && keep && x != WX_ROOT ? prefix_rank(Fs, 0, Cs, P.c_shift, x) : x;
+            en[r] = (p << 24) | low;
             kept[r] = __ballot_sync(0xFFFFFFFFu, keep);
         }
         uint32_t tot = 0;
@@ -381,14 +393,16 @@ __global__ void __launch_bounds__((TB == WT_L2 ? WNW_SMALL : WNW) * 32, 1)
     const uint32_t gw = blockIdx.x * NW + warp, gstride = gridDim.x * NW;
     if (blockIdx.x * NW >= n_pairs) return;
 
-    // shared memory: H (all copies), the prefix bitmap, the queues
+    // shared memory: H (all copies), the prefix bitmap and its counts, the queues
     const uint32_t hwords = TB == WT_L2 ? 0u : P.w_words << P.w_rep;
     uint32_t *Fs = reinterpret_cast<uint32_t *>(smem) + hwords;
-    uint32_t *q = Fs + (TB == WT_L2 ? 0u : P.wf_words) + warp * WQCAP;
+    uint32_t *Cs = Fs + (TB == WT_L2 ? 0u : P.wf_words);
+    uint32_t *q = Cs + (TB == WT_L2 ? 0u : P.wc_words) + warp * WQCAP;
     if (TB != WT_L2) {
         w_fill<NW * 32>(reinterpret_cast<uint32_t *>(smem), P.T.H, P.w_words,
                         TB == WT_ONE ? 0u : P.w_rep, blockIdx.x * 160u);
         w_fill<NW * 32>(Fs, P.F, P.wf_words, 0u, blockIdx.x * 32u);
+        w_fill<NW * 32>(Cs, P.C, P.wc_words, 0u, 0u);
         __syncthreads();
     }
     // from here on the call's counters are used, zeroed by the kernel before
@@ -400,7 +414,7 @@ __global__ void __launch_bounds__((TB == WT_L2 ? WNW_SMALL : WNW) * 32, 1)
     K.hm = TB == WT_COPIES ? P.w_words << (2 + P.w_rep) : P.w_words;
     K.amask = ~((4u << P.w_rep) - 1u);
     K.c4 = (lane & ((1u << P.w_rep) - 1u)) << 2;
-    const uint32_t *Fq = (TB != WT_L2 && P.wf_words) ? Fs : nullptr;
+    const uint32_t *Fq = (TB != WT_L2 && P.wf_words) ? Fs : nullptr, *Cq = Cs;
 
     const uint64_t N = P.n, N16 = N & ~15ull;
     const uint32_t lt = (1u << lane) - 1u;
@@ -496,7 +510,7 @@ __global__ void __launch_bounds__((TB == WT_L2 ? WNW_SMALL : WNW) * 32, 1)
             qn += __popc(any);
             if (qn > WQCAP - 32 || i >= n_it) {
                 __syncwarp();
-                w_flush<PACKED, S>(P, q, qn, Fq, gw, gstride, lane);
+                w_flush<PACKED, S>(P, q, qn, Fq, Cq, gw, gstride, lane);
                 qn = 0;
             }
             any = __ballot_sync(0xFFFFFFFFu, m != 0);
@@ -589,7 +603,7 @@ __global__ void __launch_bounds__(RES_WARPS * 32, RES_CTAS)
         // 2 stopped on merged leaf st, 3 output known (fin)
         int state[WRU];
         uint32_t unit[WRU], pos[WRU], lim[WRU], st[WRU], q[WRU], fin[WRU], tq[WRU], t0[WRU], t1[WRU];
-        uint32_t slo[WRU], shi[WRU], x[WRU], slot[WRU];
+        uint32_t slo[WRU], x[WRU], slot[WRU], tn[WRU];
 #pragma unroll
         for (int u = 0; u < WRU; u++) {
             const uint32_t e = b + 32 * u + lane;
@@ -613,20 +627,17 @@ __global__ void __launch_bounds__(RES_WARPS * 32, RES_CTAS)
             }
             // the slice's first offset indices, the text from p + k on (from
             // p for a walk from the root)
-            slo[u] = shi[u] = 0;
-            if (P.n_seg > 1) {
-                slo[u] = __ldg(P.unit_seg + unit[u]);
-                shi[u] = unit[u] + 1 < P.n_tiles ? __ldg(P.unit_seg + unit[u] + 1) : P.n_seg;
-            }
+            slo[u] = P.n_seg > 1 ? __ldg(P.unit_seg + unit[u]) : 0u;
             tq[u] = pos[u] + (x[u] == WX_ROOT ? 0u : k);
-            const uint64_t a = ((uint64_t)unit[u] << SLICE_SHIFT) + tq[u], c = a & ~3ull;
-            const bool ok = on && c + 12 <= P.n;
+            // the aligned 8-byte piece, and the next where it holds few of them
+            const uint64_t a = ((uint64_t)unit[u] << SLICE_SHIFT) + tq[u], c = a & ~7ull;
+            const bool ok = on && c + 16 <= P.n, two = ok && ((uint32_t)a & 7u) > 4;
             const uint8_t *src = P.in + (ok ? c : 0ull);
-            const uint32_t w0 = ld_stream4_if(ok, src), w1 = ld_stream4_if(ok, src + 4),
-                           w2 = ld_stream4_if(ok, src + 8);
-            const uint32_t sh = 8 * ((uint32_t)a & 3u);
-            t0[u] = __funnelshift_r(w0, w1, sh);
-            t1[u] = __funnelshift_r(w1, w2, sh);
+            const uint2 pa = ld_stream8_if(ok, src), pb = ld_stream8_if(two, src + 8);
+            const uint2 s8 = bytes8(make_uint4(pa.x, pa.y, pb.x, pb.y), (uint32_t)a & 7u);
+            t0[u] = s8.x;
+            t1[u] = s8.y;
+            tn[u] = two ? 8u : 8u - ((uint32_t)a & 7u);
             if (!ok) tq[u] = 0xFFFFFF00u;  // no symbol at hand
         }
 #pragma unroll
@@ -635,13 +646,21 @@ __global__ void __launch_bounds__(RES_WARPS * 32, RES_CTAS)
             const uint64_t remain = P.n - us;
             lim[u] = remain < LIM_MAX ? (uint32_t)remain : LIM_MAX;
             if (P.n_seg > 1) {
+                // the first offset beyond p, from the slice's first index on:
+                // a few steps, then by search up to the next slice's index
                 // (bounded: offsets out of order leave some indices unwritten)
-                uint32_t lo = slo[u] < P.n_seg ? slo[u] : P.n_seg, hi = shi[u] < P.n_seg ? shi[u] : P.n_seg;
-                while (lo < hi) {
-                    const uint32_t mid = (lo + hi) >> 1;
-                    if (__ldg(P.seg + mid) > p) hi = mid; else lo = mid + 1;
+                uint32_t lo = slo[u] < P.n_seg ? slo[u] : P.n_seg;
+                uint64_t e = __ldg(P.seg + lo);
+                for (uint32_t i = 0; i < 3 && e <= p && lo < P.n_seg; i++) e = __ldg(P.seg + ++lo);
+                if (e <= p && lo < P.n_seg) {
+                    uint32_t hi = unit[u] + 1 < P.n_tiles ? __ldg(P.unit_seg + unit[u] + 1) : P.n_seg;
+                    hi = hi < P.n_seg ? hi : P.n_seg;
+                    while (lo < hi) {
+                        const uint32_t mid = (lo + hi) >> 1;
+                        if (__ldg(P.seg + mid) > p) hi = mid; else lo = mid + 1;
+                    }
+                    e = __ldg(P.seg + lo);
                 }
-                const uint64_t e = __ldg(P.seg + lo);
                 const uint64_t r = e > us ? e - us : 0;
                 lim[u] = r < lim[u] ? (uint32_t)r : lim[u];
             }
@@ -650,9 +669,10 @@ __global__ void __launch_bounds__(RES_WARPS * 32, RES_CTAS)
             if (DENSE) {
                 if (x[u] != WX_ROOT) q[u] += k;
             } else if (state[u] == 0 && x[u] != WX_ROOT && pos[u] + k <= lim[u]) {
-                // (the scan has tested the index's bit)
-                const uint32_t xx = (uint32_t)chk(P, x[u], 1ull << (k * P.T.bps));
-                const uint32_t r = (uint32_t)chk(P, prefix_rank(P.F, 0, P.C, P.c_shift, xx), P.T.n_e[k]);
+                // (the scan has tested the index's bit, or ranked it too)
+                uint32_t r = x[u];
+                if (!P.w_ranked) r = prefix_rank(P.F, 0, P.C, P.c_shift, (uint32_t)chk(P, r, 1ull << (k * P.T.bps)));
+                r = (uint32_t)chk(P, r, P.T.n_e[k]);
                 const uint32_t ev = __ldg(P.E + r);
                 q[u] = pos[u] + k;
                 if (ev & D_CONT) {
@@ -667,7 +687,7 @@ __global__ void __launch_bounds__(RES_WARPS * 32, RES_CTAS)
         auto symbol = [&](int u, uint32_t i) -> uint32_t {
             if (i >= lim[u]) return 0x100u;
             const uint32_t d = i - tq[u];
-            if (d < 8) return ((d < 4 ? t0[u] : t1[u]) >> (8 * (d & 3))) & 0xFFu;
+            if (d < tn[u]) return ((d < 4 ? t0[u] : t1[u]) >> (8 * (d & 3))) & 0xFFu;
             return __ldg(P.in + chk(P, ((uint64_t)unit[u] << SLICE_SHIFT) + i, P.n));
         };
         // ---- three rounds, one record of each walk a round

@@ -384,7 +384,7 @@ struct Plan {
     // plan that its options would otherwise run): words of the prefix bitmap
     // in its shared memory
     bool win;
-    uint32_t wf_words;
+    uint32_t wf_words, wc_words;
     size_t smem_win;
     void *kernel_win, *kernel_win_small;
     // the dense scan kernel takes it: its tables in shared memory
@@ -962,8 +962,12 @@ static int make_plan(const pfac_table *t, uint32_t n_seg, const pfac_match_opts 
     const size_t fixed = ((size_t)T.w_words << T.w_rep) * 4 + WNW * WQCAP * 4;
     if (fixed > SMEM_LIMIT) return PFAC_OK;
     const uint64_t fw = ((1ull << (pl->k * T.bps)) + 31) / 32;
-    if (fw % 4 == 0 && fixed + fw * 4 <= SMEM_LIMIT) pl->wf_words = (uint32_t)fw;
-    pl->smem_win = fixed + (size_t)pl->wf_words * 4;
+    const uint64_t cw = (fw + (1ull << T.c_shift[pl->k]) - 1) >> T.c_shift[pl->k];
+    if (fw % 4 == 0 && cw % 4 == 0 && fixed + (fw + cw) * 4 <= SMEM_LIMIT) {
+        pl->wf_words = (uint32_t)fw;
+        pl->wc_words = (uint32_t)cw;
+    }
+    pl->smem_win = fixed + ((size_t)pl->wf_words + pl->wc_words) * 4;
     pl->kernel_win = scan_kernel_w(T, T.w_rep ? WT_COPIES : WT_ONE);
     pl->kernel_win_small = scan_kernel_w(T, WT_L2);
     pl->kernel_res = wresolve_kernel((int)T.W);
@@ -1219,6 +1223,7 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
         P.w_glen = T.w_glen;
         P.w_badmask = T.w_short ? 0x01010101u * ((0xFFu << T.bps) & 0xFFu) : 0u;
         P.wf_words = pl.wf_words;
+        P.wc_words = pl.wc_words;
         P.unordered = 1;
         P.chunk_adds = P.chunk_shift == CHUNK_SHIFT_MIN;
     } else if (pl.defer && !pl.dsc) {
@@ -1263,6 +1268,7 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
         // few pairs of slices: one warp each, the filter read through L2
         const uint32_t n_pairs = (P.n_tiles + 1) / 2;
         const bool small = n_pairs <= (uint32_t)nsm * WIN_SMALL_PAIRS;
+        P.w_ranked = !small && P.wf_words != 0;
         const uint32_t nw = small ? WNW_SMALL : WNW;
         const uint32_t need = (n_pairs + nw - 1) / nw;
         void *args[] = {&P};

@@ -63,6 +63,12 @@ bool build_window_filter(const std::vector<WinPat> &pats, uint32_t sigma, uint32
             }
         }
     }
+    // powers of the symbol counts
+    std::vector<double> a_pow(64, 1.0), s_pow(64, 1.0);
+    for (int i = 1; i < 64; i++) {
+        a_pow[i] = a_pow[i - 1] * A;
+        s_pow[i] = s_pow[i - 1] / (double)sigma;
+    }
     double best = MAX_COST;
     bool found = false;
     for (const Shape &s : shapes) {
@@ -76,9 +82,9 @@ bool build_window_filter(const std::vector<WinPat> &pats, uint32_t sigma, uint32
             if (!by_len[L]) continue;
             for (uint32_t o = 0; o < s.S; o++) {
                 const uint32_t known = L > o ? std::min(L - o, glen) : 0u;
-                const double n = by_len[L] * pow(A, (double)(glen - known));
+                const double n = by_len[L] * a_pow[glen - known];
                 ins += n;
-                real += by_len[L] * pow((double)sigma, -(double)known);
+                real += by_len[L] * s_pow[known];
                 if (!packed && known < glen && known >= s.gw) full += by_len[L];
             }
         }
@@ -100,12 +106,14 @@ bool build_window_filter(const std::vector<WinPat> &pats, uint32_t sigma, uint32
                 if (mu > 30.0) {
                     fp = pow(1.0 - pow(31.0 / 32.0, mu * s.nb), (double)s.nb);
                 } else {
-                    double pn = exp(-mu);
+                    double pn = exp(-mu), clear = 1.0;  // clear: a bit none of n strings set
+                    const double keep = s.nb == 2 ? 961.0 / 1024.0 : 29791.0 / 32768.0;  // (31/32)^nb
                     for (int n = 0; n < 200; n++) {
-                        const double set = 1.0 - pow(31.0 / 32.0, n * (double)s.nb);
-                        fp += pn * pow(set, (double)s.nb);
+                        const double set = 1.0 - clear;
+                        fp += pn * (s.nb == 2 ? set * set : set * set * set);
                         pn *= mu / (n + 1);
-                        if (n > mu && pn < 1e-12) break;
+                        clear *= keep;
+                        if (n > mu && pn < 1e-9) break;
                     }
                 }
                 if (full > 0) fp += 1.0 - exp(-full / words);
