@@ -5,7 +5,7 @@
 // Nearly every candidate is a match here, so what counts is the work per
 // match, not the filter.  A warp takes chunks of 1,024 bytes (two slices); a
 // lane packs its 32 symbols into two words and tests 32 prefix indices against
-// the prefix bitmap F_k (copies over the banks).  The slice's candidates are
+// the prefix bitmap F_k (copies over the banks).  The chunk's candidates are
 // listed in shared memory in position order, then taken 32 at a time, one per
 // lane: rank in F_k, entry E_k (in shared memory where it fits), and the
 // record, stored coalesced at the candidate's rank in its slice.  An entry
@@ -18,9 +18,10 @@
 //
 // 128 MiB over 4 symbols with 1,000 patterns of 4 to 64 symbols (one position
 // in twelve matches): the queued kernel, which resolved every candidate from
-// its queue through L2, took 760 us; this one 206 us, and 43 us for the pending
-// records.  It is bound by the instructions per position and per candidate (68%
-// issue, 70% of the ALU pipe).
+// its queue through L2, took 760 us; this one 162 us, and 43 us for the pending
+// records (206 us when each slice listed its candidates by itself, with half
+// the lanes idle).  It is bound by the instructions per position and per
+// candidate (68% issue, 70% of the ALU pipe at 206 us).
 #pragma once
 #include "kernels_w.cuh"
 
@@ -29,7 +30,7 @@ namespace pfac {
 constexpr int DNW = 24;               // warps per CTA
 constexpr uint32_t DQCAP = 64;        // pending records queued per warp
 struct DWarpArea {
-    uint32_t list[SLICE];             // candidates: position | symbols << 9 | D_LIST_ROOT
+    uint32_t list[2 * SLICE];         // candidates: position | symbols << 10 | D_LIST_ROOT
     uint32_t pend[DQCAP];             // chunk << 10 | slice << 9 | slot
 };
 constexpr uint32_t D_LIST_ROOT = 0x80000000u;
@@ -163,87 +164,91 @@ __global__ void __launch_bounds__(DNW * 32, 1) k_scand(const __grid_constant__ M
             const uint64_t left = P.starts_end > o ? P.starts_end - o : 0;
             m &= left >= 32 ? 0xFFFFFFFFu : (1u << (uint32_t)left) - 1u;
         }
-        // ---- each slice: its lanes' candidates listed in position order
-        uint32_t incl = __popc(m);
-        const uint32_t own_n = incl;
+        // ---- the chunk's candidates listed in position order
+        uint32_t at = __popc(m);
+        const uint32_t own_n = at;
 #pragma unroll
-        for (int s = 1; s < 16; s <<= 1) {
-            const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, s, 16);
-            if ((lane & 15) >= (uint32_t)s) incl += v;
+        for (int s = 1; s < 32; s <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, at, s);
+            if (lane >= (uint32_t)s) at += v;
         }
-#pragma unroll 1
-        for (uint32_t s = 0; s < 2; s++) {
-            const uint64_t u = 2 * g + s;
-            if (u >= P.n_tiles) break;
-            const uint32_t tot = __shfl_sync(0xFFFFFFFFu, incl, 16 * s + 15);
-            if (tot == 0) continue;
-            if ((lane >> 4) == s) {
-                uint32_t mm = m, at = incl - own_n;
-                while (mm) {
-                    const uint32_t j = __ffs(mm) - 1;
-                    mm &= mm - 1;
-                    const uint32_t lo = j < 16 ? w0 : w1, hi = j < 16 ? w1 : w2;
-                    const uint32_t t = __funnelshift_r(lo, hi, 2 * (j & 15)) & ((1u << (2 * D_LIST_SYMS)) - 1u);
-                    A.list[at++] = ((lane & 15) * 32 + j) | (t << 9) | (((root >> j) & 1u) ? D_LIST_ROOT : 0u);
-                }
-            }
-            __syncwarp();
-            uint64_t *rec = P.recs + (size_t)u * P.unit_cap;
-            uint32_t keys = 0;
-            for (uint32_t b0 = 0; b0 < tot; b0 += 32) {
-                const uint32_t idx = b0 + lane;
-                bool pend = false;
-                uint32_t fin = 0, pos = 0;
-                if (idx < tot) {
-                    const uint32_t e = A.list[idx];
-                    pos = e & (SLICE - 1);
-                    if (e & D_LIST_ROOT) {
+        const uint32_t tot_a = __shfl_sync(0xFFFFFFFFu, at, 15), tot = __shfl_sync(0xFFFFFFFFu, at, 31);
+        at -= own_n;
+        uint32_t mm = m;
+        while (mm) {
+            const uint32_t j = __ffs(mm) - 1;
+            mm &= mm - 1;
+            const uint32_t lo = j < 16 ? w0 : w1, hi = j < 16 ? w1 : w2;
+            const uint32_t t = __funnelshift_r(lo, hi, 2 * (j & 15)) & ((1u << (2 * D_LIST_SYMS)) - 1u);
+            A.list[at++] = (lane * 32 + j) | (t << 10) | (((root >> j) & 1u) ? D_LIST_ROOT : 0u);
+        }
+        __syncwarp();
+        // the records of both slices, 32 candidates at a time (no candidate of
+        // the second where it lies past the last unit)
+        const uint64_t u0 = 2 * g;
+        uint32_t keys_a = 0, keys_b = 0;
+        for (uint32_t b0 = 0; b0 < tot; b0 += 32) {
+            const uint32_t idx = b0 + lane;
+            bool pend = false;
+            const bool second = idx >= tot_a;
+            const uint32_t slot = second ? idx - tot_a : idx;
+            if (idx < tot) {
+                const uint32_t e = A.list[idx];
+                const uint64_t u = u0 + (second ? 1 : 0);
+                uint32_t fin, keys = 0;
+                if (e & D_LIST_ROOT) {
+                    pend = true;
+                    fin = D_PEND | D_PEND_ROOT;
+                } else {
+                    const uint32_t t = (e & ~D_LIST_ROOT) >> 10;
+                    const uint32_t x = t & kmask;
+                    const uint32_t r = (uint32_t)chk(
+                        P, prefix_rank(Fs + (rep ? copy : 0u), rep, Cs, P.c_shift, x), P.T.n_e[k]);
+                    const uint32_t ev = ES ? Es[r] : __ldg(P.E + r);
+                    if (ev & D_CONT) {
                         pend = true;
-                        fin = D_PEND | D_PEND_ROOT;
-                    } else {
-                        const uint32_t t = (e & ~D_LIST_ROOT) >> 9;
-                        const uint32_t x = t & kmask;
-                        const uint32_t r = (uint32_t)chk(
-                            P, prefix_rank(Fs + (rep ? copy : 0u), rep, Cs, P.c_shift, x), P.T.n_e[k]);
-                        const uint32_t ev = ES ? Es[r] : __ldg(P.E + r);
-                        if (ev & D_CONT) {
-                            pend = true;
-                            if (P.tbl_m_words && k < D_LIST_SYMS) {
-                                // four mask bits an entry (all: it reports output)
-                                const uint32_t mr = (Ms[r >> 3] >> (4 * (r & 7))) & 15u;
-                                const uint32_t c = (t >> (2 * k)) & 3u;
-                                pend = mr == 15u || (c < sigma && ((mr >> c) & 1u));
-                            }
-                            fin = pend ? D_PEND | (ev & D_PEND_STATE) : 0u;
-                        } else {
-                            // (long lists are counted on their own: the sum
-                            // of the others stays in 32 bits)
-                            fin = ev;
-                            if ((ev & FIN_LEN_ESC) != FIN_LEN_ESC) keys += ev & FIN_LEN_ESC;
-                            else atomicAdd((unsigned long long *)(P.tile_k + u),
-                                           (unsigned long long)fin_len_c(P, ev));
+                        if (P.tbl_m_words && k < D_LIST_SYMS) {
+                            // four mask bits an entry (all: it reports output)
+                            const uint32_t mr = (Ms[r >> 3] >> (4 * (r & 7))) & 15u;
+                            const uint32_t c = (t >> (2 * k)) & 3u;
+                            pend = mr == 15u || (c < sigma && ((mr >> c) & 1u));
                         }
-                    }
-                    rec[idx] = ((uint64_t)pos << 32) | fin;
-                }
-                const uint32_t pm = __ballot_sync(0xFFFFFFFFu, pend);
-                if (pm) {
-                    if (pend) A.pend[np + __popc(pm & lt)] = (i << 10) | (s << 9) | idx;
-                    np += __popc(pm);
-                    if (np > DQCAP - 32) {
-                        __syncwarp();
-                        d_flush(P, A.pend, np, gw, gstride, lane);
-                        np = 0;
+                        fin = pend ? D_PEND | (ev & D_PEND_STATE) : 0u;
+                    } else {
+                        // (long lists are counted on their own: the sum of
+                        // the others stays in 32 bits)
+                        fin = ev;
+                        if ((ev & FIN_LEN_ESC) != FIN_LEN_ESC) keys = ev & FIN_LEN_ESC;
+                        else atomicAdd((unsigned long long *)(P.tile_k + u),
+                                       (unsigned long long)fin_len_c(P, ev));
                     }
                 }
+                keys_a += second ? 0u : keys;
+                keys_b += second ? keys : 0u;
+                P.recs[(size_t)u * P.unit_cap + slot] = ((uint64_t)(e & (SLICE - 1)) << 32) | fin;
             }
-            keys = __reduce_add_sync(0xFFFFFFFFu, keys);
-            if (lane == 0) {
-                P.tile_m[u] = tot;
-                atomicAdd((unsigned long long *)(P.tile_k + u), (unsigned long long)keys);
+            const uint32_t pm = __ballot_sync(0xFFFFFFFFu, pend);
+            if (pm) {
+                if (pend) A.pend[np + __popc(pm & lt)] = (i << 10) | (second ? (uint32_t)SLICE : 0u) | slot;
+                np += __popc(pm);
+                if (np > DQCAP - 32) {
+                    __syncwarp();
+                    d_flush(P, A.pend, np, gw, gstride, lane);
+                    np = 0;
+                }
             }
-            __syncwarp();
         }
+        keys_a = __reduce_add_sync(0xFFFFFFFFu, keys_a);
+        keys_b = __reduce_add_sync(0xFFFFFFFFu, keys_b);
+        if (lane < 2) {
+            const uint32_t n = lane ? tot - tot_a : tot_a;
+            if (n) {
+                P.tile_m[u0 + lane] = n;
+                atomicAdd((unsigned long long *)(P.tile_k + u0 + lane),
+                          (unsigned long long)(lane ? keys_b : keys_a));
+            }
+        }
+        __syncwarp();
         c0 = c1;
         h0 = h1;
     }
