@@ -40,7 +40,6 @@ sys.path.insert(0, ROOT)
 
 import workloads  # noqa: E402
 
-SCAN_KERNELS_PER_STEP = 5  # scan, key-count reduce, offsets, overflow re-scan, key expansion
 # (plus the resolver kernel where the plan hands queues over)
 
 
@@ -85,6 +84,24 @@ def kernel_digest():
             if code:
                 h.update(code.encode() + b"\n")
     return h.hexdigest()[:16]
+
+
+def spelt_workspace(pfac, table, n_bytes, n_seg, plan):
+    """Workspace of a call with the plan's scan kernel, resolver and records
+    fixed by its options."""
+    return pfac.workspace_bytes(table, n_bytes, n_seg, scan_kernel=plan["scan_kernel"],
+                                resolver=plan["resolver"], records_per_slice=plan["records_per_slice"])
+
+
+def launches_per_step(pfac, table, n_bytes, n_seg, plan, opt):
+    """This library's kernel launches of one match call.  A call that takes the
+    window or dense scan kernel (its workspace then differs from the one of
+    the plan spelt out) clears, scans, resolves and expands, and sums chunk
+    counts beyond 65,536 slices; any other scans, sums, expands and emits,
+    with the resolver and the segment pass where the plan has them."""
+    if pfac.workspace_bytes(table, n_bytes, n_seg, **opt) != spelt_workspace(pfac, table, n_bytes, n_seg, plan):
+        return 4 + (1 if n_bytes > (65536 << 9) else 0)
+    return 4 + (1 if plan["resolver"] == 2 else 0) + (1 if n_seg > 1 else 0)
 
 
 def measured_traffic(workload, plan):
@@ -433,7 +450,10 @@ def time_cell(pfac, torch, w, dev, stream, args, user_opt, workload_name, graph_
                 "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)",
                 "traffic": args.traffic if (args.traffic is not None and graph_steps) else (
                     measured_traffic(workload_name, plan) if not user_opt else None),
-                "kernel": "k_scanq (compressed-table scan: scan pass + emit pass)",
+                "kernel": ("k_scanw or k_scand with k_wresolve (compressed-table scan and its resolver)"
+                           if pfac.workspace_bytes(table, N, S, **user_opt) != spelt_workspace(
+                               pfac, table, N, S, plan) else
+                           "k_scanq or k_scanr (compressed-table scan: scan pass + emit pass)"),
                 "alg_bytes_per_launch": alg_bytes,
                 "scan_pass_ms": round(scan_avg_ms, 4), "emit_pass_ms": round(emit_avg_ms, 4)}
     cell = {
@@ -454,6 +474,7 @@ def time_cell(pfac, torch, w, dev, stream, args, user_opt, workload_name, graph_
         "build_s": {"compressed": round(build_s, 3), "dense": round(dense_build_s, 3)},
         "roofline": roofline,
         "scan_plan": plan, "autotuned": tune, "cuda_graph": bool(graph is not None),
+        "launches_per_step": launches_per_step(pfac, table, N, S, plan, user_opt),
         "wall_s_timed": round(wall, 4),
         "clocks": clk,
     }
@@ -660,11 +681,7 @@ def run_ours(args):
         extra["serving"] = serving_levels(args, [100.0], 2.0, 30, 2000, verbose=False)[0]
 
     roofline = cell.pop("roofline")
-    # this library's launches per step: the five of every call, the resolver
-    # kernel where the plan hands queues to it, the segment pass for several
-    # segments
-    per_step = SCAN_KERNELS_PER_STEP + (1 if cell["scan_plan"].get("resolver") == 2 else 0) + \
-        (1 if S > 1 else 0)
+    per_step = cell.pop("launches_per_step")
     line = {
         "metric": METRIC,
         "value": round(value, 3), "unit": "Gbps", "n_gpus": world, "steps": K, "warmup": W,
