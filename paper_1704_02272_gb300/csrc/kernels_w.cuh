@@ -23,21 +23,20 @@
 //   call's entry buffer with one atomic, on one of up to 64 parts of it so
 //   that the warps do not queue on one counter.  When a part is full its
 //   warps' lanes walk their starts from the root instead.
-// * k_wresolve then takes the entries in any order: segment limit, exact
-//   prefix bit, the batched walks of the queued kernel's resolver, and one
-//   record per match at an atomically taken slot of its slice; the key
-//   expansion sorts the few records of a slice.
+// * k_wresolve then takes the entries in any order: segment limit, prefix
+//   entry, the walk, and one record per match at an atomically taken slot of
+//   its slice; the key expansion sorts the few records of a slice.
 //
 // What bounds it: shared-memory lookups (3.7 wavefronts of random banks per
 // warp-wide lookup with one copy of H: 59 cycles of an SM's shared memory per
 // slice at stride 1) and the ALU instructions around them; S, the bits tested
 // and the copies of H are chosen per table to balance both (window.cpp).
 // Measured scan pass, before (queued or register-staged kernel) and with this
-// one: 20 symbols x 10,000 patterns, 256 MiB: 858 -> 184 us; 64 x 100,000,
-// 128 MiB: 569 -> 118 us; 256 x 1,000, 512 MiB: 293 -> 200 us; 52 letters x
+// one: 20 symbols x 10,000 patterns, 256 MiB: 858 -> 174 us; 64 x 100,000,
+// 128 MiB: 569 -> 108 us; 256 x 1,000, 512 MiB: 293 -> 159 us; 52 letters x
 // 100, 100 MiB: 111 -> 32 us; 1 GiB of packets against 20,000 signatures:
-// 2,773 -> 878 us; DNA x 10,000, 256 MiB: 281 -> 182 us.  The resolver after
-// it takes the place of the other kernels' resolver (packets: 374 -> 363 us).
+// 2,773 -> 781 us; DNA x 10,000, 256 MiB: 281 -> 185 us.  The resolver after
+// it takes the place of the other kernels' resolver (packets: 374 -> 297 us).
 #pragma once
 #include "kernels_r.cuh"
 
