@@ -24,8 +24,19 @@ constexpr double WAVEFRONTS[6] = {3.7, 3.4, 3.1, 2.85, 2.0, 1.0};
 
 // Most strings inserted (completions of short patterns included).
 constexpr double MAX_STRINGS = 2.0e6;
-// Estimated SM cycles per slice above which the other scan kernels are used.
-constexpr double MAX_COST = 600.0;
+// Estimated SM cycles per slice above which the other scan kernels are used:
+// one line for alphabets of 17 symbols on, one below.  64 MiB of uniform text,
+// patterns of 4 to 64 symbols, this kernel / the faster of the others (the
+// estimate): 20 symbols x 100,000 398 / 2,607 us (356); 256 x 100,000 93 / 331
+// (150); 64 x 300,000 324 / 2,556 (781); 64 x 500,000 646 / 3,004 (1,850);
+// 256 x 500,000 595 / 1,029 (1,816); 256 x 1,000,000 1,231 / 2,049 (3,680); 20
+// x 300,000 from 6 symbols on 922 / 3,787 (726).  Packets, 50,000 signatures:
+// 232 / 532 (422).  Small alphabets, whose few hashed symbols say less while
+// the other kernels' filters see more of them: 4 x 300,000 from 14 symbols on
+// 215 / 1,086 (494), but 10 x 20,000 from 5 on 733 / 599 (640) and 8 x 30,000
+// from 6 on 1,304 / 234 (2,398).
+constexpr double MAX_COST = 4000.0;
+constexpr double MAX_COST_SMALL = 600.0;  // up to 16 symbols
 
 struct Shape {
     uint32_t S, gw, g5, nb;
@@ -69,7 +80,7 @@ bool build_window_filter(const std::vector<WinPat> &pats, uint32_t sigma, uint32
         a_pow[i] = a_pow[i - 1] * A;
         s_pow[i] = s_pow[i - 1] / (double)sigma;
     }
-    double best = MAX_COST;
+    double best = bps > 4 ? MAX_COST : MAX_COST_SMALL;
     bool found = false;
     for (const Shape &s : shapes) {
         uint32_t glen = s.gw;

@@ -176,3 +176,14 @@ def test_graph_replay_on_changed_text():
             x = workloads.Workload("g", 52, w.patterns, data, w.seg_offsets)
             assert int(st.item()) == 0
             assert_same(keys_np(out[:int(cnt.item())]), oracle_keys(x), "replay")
+
+
+@pytest.mark.parametrize("n_bytes", [30_011, 3_000_017])
+def test_crowded_filters(n_bytes):
+    # sets so large that most words of the filter hold bits and many windows
+    # pass: the entry buffer's parts fill up
+    for sigma, n, lo, hi in ((17, 200_000, 6, 8), (64, 260_000, 4, 5)):
+        w = workloads.tiny_case(7900 + sigma, sigma, n, lo, hi, n_bytes, n_segments=7,
+                                n_plants=20 + n_bytes // 500)
+        with pfac.Table(w.patterns, sigma) as t:
+            check(t, w, f"{sigma} symbols, {n} patterns, {n_bytes} bytes")
