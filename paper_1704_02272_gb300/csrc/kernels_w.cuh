@@ -158,16 +158,23 @@ __device__ __forceinline__ void w_emit(const MatchParams &P, uint32_t u, uint32_
 
 // Walk limit of start p of slice u, relative to the slice start: the first
 // offset above p, found between the slice's first offset index and the next
-// slice's.
+// slice's (INDEXED), or among all offsets.  The indices are written by the
+// scan launch itself, each by any of its warps, so that only the launches
+// after it may read them.
+template <bool INDEXED>
 __device__ __forceinline__ uint32_t w_limit(const MatchParams &P, uint32_t u, uint64_t p) {
     const uint64_t ustart = (uint64_t)u << SLICE_SHIFT;
     const uint64_t remain = P.n - ustart;
     const uint32_t rem = remain < LIM_MAX ? (uint32_t)remain : LIM_MAX;
     if (P.n_seg <= 1) return rem;
-    // (bounded: offsets out of order leave some indices unwritten)
-    uint32_t lo = __ldg(P.unit_seg + u), hi = u + 1 < P.n_tiles ? __ldg(P.unit_seg + u + 1) : P.n_seg;
-    lo = lo < P.n_seg ? lo : P.n_seg;
-    hi = hi < P.n_seg ? hi : P.n_seg;
+    uint32_t lo = 1, hi = P.n_seg;
+    if (INDEXED) {
+        // (bounded: offsets out of order leave some indices unwritten)
+        lo = __ldg(P.unit_seg + u);
+        hi = u + 1 < P.n_tiles ? __ldg(P.unit_seg + u + 1) : P.n_seg;
+        lo = lo < P.n_seg ? lo : P.n_seg;
+        hi = hi < P.n_seg ? hi : P.n_seg;
+    }
     while (lo < hi) {
         const uint32_t mid = (lo + hi) >> 1;
         if (__ldg(P.seg + mid) > p) hi = mid; else lo = mid + 1;
@@ -177,7 +184,8 @@ __device__ __forceinline__ uint32_t w_limit(const MatchParams &P, uint32_t u, ui
     return r < rem ? (uint32_t)r : rem;
 }
 
-// A lane's walk from the root, for starts the entry buffer has no room for.
+// A lane's walk from the root, for starts the entry buffer has no room for
+// (and, after the scan, for slices whose records were not kept).
 template <int W>
 __device__ __forceinline__ uint32_t w_walk_fin(const MatchParams &P, uint64_t ub, uint32_t q,
                                                uint32_t lim) {
@@ -209,7 +217,7 @@ __device__ __forceinline__ uint32_t w_walk_any(const MatchParams &P, uint64_t ub
 static __device__ __noinline__ void w_walk(const MatchParams *PP, uint64_t p) {
     const MatchParams &P = *PP;
     const uint32_t u = (uint32_t)(p >> SLICE_SHIFT), pos = (uint32_t)p & (SLICE - 1);
-    const uint32_t fin = w_walk_any(P, (uint64_t)u << SLICE_SHIFT, pos, w_limit(P, u, p));
+    const uint32_t fin = w_walk_any(P, (uint64_t)u << SLICE_SHIFT, pos, w_limit<false>(P, u, p));
     if (fin) w_emit(P, u, pos, fin);
 }
 

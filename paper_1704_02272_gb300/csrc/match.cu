@@ -236,7 +236,7 @@ static __device__ __noinline__ void expand_unit(const MatchParams *PP, uint64_t 
         const uint32_t pos = p0 + lane;
         uint32_t fin = 0, L = 0;
         if (us + pos < P.starts_end) {
-            fin = w_walk_any(P, us, pos, w_limit(P, (uint32_t)t, us + pos));
+            fin = w_walk_any(P, us, pos, w_limit<true>(P, (uint32_t)t, us + pos));
             if (fin) L = fin_len_c(P, fin);
         }
         const uint32_t before = keys_before<32>(pos, L, false, lane);
