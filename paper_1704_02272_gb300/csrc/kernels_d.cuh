@@ -96,6 +96,9 @@ __global__ void __launch_bounds__(DNW * 32, 1) k_scand(const __grid_constant__ M
 
     const uint64_t N = P.n, N16 = N & ~15ull;
     const uint32_t k = P.k, kmask = (1u << (2 * k)) - 1u, sigma = P.T.sigma;
+    // symbols read from a start on: its window, and the next for the masks
+    const bool masks = P.tbl_m_words != 0 && k < D_LIST_SYMS;
+    const uint32_t k_read = k + (masks ? 1 : 0);
     const uint32_t lt = (1u << lane) - 1u;
     const bool l31 = lane == 31;
     const bool al32 = ((uintptr_t)P.in & 31) == 0;
@@ -145,8 +148,9 @@ __global__ void __launch_bounds__(DNW * 32, 1) k_scand(const __grid_constant__ M
             acc[j >> 3] = __funnelshift_r(acc[j >> 3], __funnelshift_r(x, x, t), 1);
         }
         uint32_t m = __byte_perm(__byte_perm(acc[0], acc[1], 0x0073), __byte_perm(acc[2], acc[3], 0x0073), 0x5410);
-        // windows that leave the whole 16-byte pieces of the input, or hold a
-        // byte outside the 2-bit range: walked from the root
+        // windows that leave the whole 16-byte pieces of the input (with the
+        // symbol after them, which the child masks are asked about), or hold
+        // a byte outside the 2-bit range: walked from the root
         uint32_t root = 0;
         const uint32_t bad = (ca.x | ca.y | ca.z | ca.w | cb.x | cb.y | cb.z | cb.w) & 0xFCFCFCFCu;
         const uint32_t badh = (h0.x | h0.y | h0.z | h0.w) & 0xFCFCFCFCu;
@@ -158,7 +162,7 @@ __global__ void __launch_bounds__(DNW * 32, 1) k_scand(const __grid_constant__ M
         }
         if (i >= n_ok)
             for (uint32_t j = 0; j < 32; j++)
-                if (o + j + k > N16) root |= 1u << j;
+                if (o + j + k_read > N16) root |= 1u << j;
         m |= root;
         if (o + 32 > P.starts_end) {  // starts at or past it start no walk
             const uint64_t left = P.starts_end > o ? P.starts_end - o : 0;
@@ -207,7 +211,7 @@ __global__ void __launch_bounds__(DNW * 32, 1) k_scand(const __grid_constant__ M
                     const uint32_t ev = ES ? Es[r] : __ldg(P.E + r);
                     if (ev & D_CONT) {
                         pend = true;
-                        if (P.tbl_m_words && k < D_LIST_SYMS) {
+                        if (masks) {
                             // four mask bits an entry (all: it reports output)
                             const uint32_t mr = (Ms[r >> 3] >> (4 * (r & 7))) & 15u;
                             const uint32_t c = (t >> (2 * k)) & 3u;
