@@ -141,19 +141,28 @@ __device__ __forceinline__ uint32_t w_filter(const uint32_t (&w)[9], const WCons
 
 // One match: a record in the slice's space while it has room (in any order),
 // and the slice's counts: records above bit UNIT_KEY_BITS of its word, keys
-// below, so that one atomic takes the slot and counts the keys.  (A slice with
-// more matches than its space is walked again by the expansion.)  With few slices
+// below, so that one atomic takes the slots and counts the keys.  (A slice
+// with more matches than its space is walked again by the expansion.)  The
+// calling lanes' matches of a slice share one atomic: where most starts match,
+// a warp's 32 lie in one or two slices and queued on its word (8 MiB of one
+// symbol that two patterns repeat: 1,602 -> 655 us a call).  With few slices
 // the chunks' key counts are added up here too; with many, neighbouring
 // matches would queue on one chunk's word (1 GiB of packets: 0.8 instead of
 // 0.36 ms), and k_reduce sums them.
 __device__ __forceinline__ void w_emit(const MatchParams &P, uint32_t u, uint32_t pos, uint32_t fin) {
     u = (uint32_t)chk(P, u, P.n_tiles);
-    const uint32_t cap = P.unit_cap;
-    const unsigned long long keys = fin_len_c(P, fin);
-    const uint32_t rank = (uint32_t)(atomicAdd((unsigned long long *)(P.tile_k + u),
-                                               (1ull << UNIT_KEY_BITS) | keys) >> UNIT_KEY_BITS);
+    const uint32_t cap = P.unit_cap, lane = threadIdx.x & 31;
+    const uint32_t same = __match_any_sync(__activemask(), u), first = __ffs(same) - 1;
+    // (lists of at most 2^24 ids: a warp's fit 32 bits)
+    const uint32_t keys = __reduce_add_sync(same, (uint32_t)fin_len_c(P, fin));
+    uint32_t rank = 0;
+    if (lane == first) {
+        rank = (uint32_t)(atomicAdd((unsigned long long *)(P.tile_k + u),
+                                    ((unsigned long long)__popc(same) << UNIT_KEY_BITS) | keys) >> UNIT_KEY_BITS);
+        if (P.chunk_adds) atomicAdd((unsigned long long *)(P.chunk + (u >> P.chunk_shift)), (unsigned long long)keys);
+    }
+    rank = __shfl_sync(same, rank, first) + __popc(same & ((1u << lane) - 1u));
     if (rank < cap) P.recs[(size_t)u * cap + rank] = ((uint64_t)pos << 32) | fin;
-    if (P.chunk_adds) atomicAdd((unsigned long long *)(P.chunk + (u >> P.chunk_shift)), keys);
 }
 
 // Walk limit of start p of slice u, relative to the slice start: the first
