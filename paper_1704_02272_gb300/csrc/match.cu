@@ -76,13 +76,19 @@ static void *scan_kernel_w(const DevTable &T, int tb) {
     }
 }
 
-// chunks of the key-count scan: the fewest units each (a power of two, 32 at
-// least) that keep their number within this
+// chunks of the key-count scan: the fewest units each (a power of two) that
+// keep their number within CHUNKS_MAX; fewer than 32 (a unit a warp at least)
+// only while all chunks' CTAs run at once.  The expansion walks a full slice
+// again with one warp, so in small calls its slices go to as many warps as
+// there are (50,000 signatures over printable text, 32 units a chunk / this
+// rule: 64 KiB 161 / 85 us, 1 MiB 164 / 92, 9 MB 337 / 302; the kernels before
+// the window path took 139, 146 and 318).
 constexpr uint32_t CHUNKS_MAX = 2048;
-constexpr uint32_t CHUNK_SHIFT_MIN = 5;
+constexpr uint32_t CHUNK_SHIFT_MIN = 3, CHUNK_SHIFT_ADDS = 5;
+constexpr uint32_t CHUNKS_AT_ONCE = 1216;  // 152 SMs x 8
 static uint32_t chunk_shift(uint64_t n_units) {
     uint32_t s = CHUNK_SHIFT_MIN;
-    while (((n_units + (1ull << s) - 1) >> s) > CHUNKS_MAX) s++;
+    while (((n_units + (1ull << s) - 1) >> s) > (s < CHUNK_SHIFT_ADDS ? CHUNKS_AT_ONCE : CHUNKS_MAX)) s++;
     return s;
 }
 
@@ -1229,7 +1235,7 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
         P.wf_words = pl.wf_words;
         P.wc_words = pl.wc_words;
         P.unordered = 1;
-        P.chunk_adds = P.chunk_shift == CHUNK_SHIFT_MIN;
+        P.chunk_adds = P.chunk_shift <= CHUNK_SHIFT_ADDS;
     } else if (pl.defer && !pl.dsc) {
         P.defer = (uint4 *)(W + L.defer);
         P.defer_cap = L.defer_cap;
