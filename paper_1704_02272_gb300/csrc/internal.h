@@ -46,12 +46,14 @@ void clear_error();
 // with another GPU's pointers.
 int check_table_device(const pfac_table *t, void *cuda_stream, const char *who);
 
-// Stream-ordered scratch from the library's own pool of the current device
-// (freed with cudaFreeAsync), and giving back what the pool keeps.
+// Stream-ordered scratch from the library's own pool of the current context
+// (freed with cudaFreeAsync), and giving back what the pool keeps (waits for
+// the device first; nothing where there is no pool).
 cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st);
 void scratch_trim();
 
-// The current CUDA context (nullptr when it cannot be told).
-void *current_context();
+// Id of the current CUDA context, one that no other context of the process
+// has or gets (0 when it cannot be told).
+uint64_t current_context_id();
 
 }  // namespace pfac

@@ -25,45 +25,43 @@ namespace {
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
-// Per device: the CUDA context the address was looked up in, and the
-// address.  A device whose context was destroyed and created again (a
+// Per device: the id of the CUDA context the address was looked up in, and
+// the address.  A device whose context was destroyed and created again (a
 // cudaDeviceReset) gets a new lookup when its current context differs.
 struct ScratchAddr {
-    void *ctx = nullptr;
+    uint64_t ctx = 0;
     void *ptr = nullptr;
 };
 ScratchAddr g_scratch[kMaxDevices];
 
-// The driver's cuCtxGetCurrent, reached through the runtime so the library
-// needs no link against the driver library; nullptr when unavailable.
-typedef int (*CtxGetCurrentFn)(void **);
-CtxGetCurrentFn ctx_get_current() {
-    static CtxGetCurrentFn fn = [] {
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &f, 12000, cudaEnableDefault,
-                                             &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess) {
-            cudaGetLastError();
-            f = nullptr;
-        }
-        return (CtxGetCurrentFn)f;
-    }();
-    return fn;
+// An entry point of the driver library, reached through the runtime so the
+// library needs no link against it; nullptr when unavailable.
+template <class Fn>
+Fn driver_entry(const char *name) {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion(name, &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+        cudaGetLastError();
+        f = nullptr;
+    }
+    return (Fn)f;
 }
 
 }  // namespace
 
-void *pfac::current_context() {
+uint64_t pfac::current_context_id() {
+    static const auto get_current = driver_entry<int (*)(void **)>("cuCtxGetCurrent");
+    static const auto get_id = driver_entry<int (*)(void *, unsigned long long *)>("cuCtxGetId");
     void *ctx = nullptr;
-    CtxGetCurrentFn f = ctx_get_current();
-    if (!f || f(&ctx) != 0) return nullptr;
-    return ctx;
+    unsigned long long id = 0;
+    if (!get_current || !get_id || get_current(&ctx) != 0 || !ctx || get_id(ctx, &id) != 0) return 0;
+    return id;
 }
 
 namespace {
 
-using pfac::current_context;
+using pfac::current_context_id;
 
 // Device address of this device's copy of the array.  In host code the
 // array's name is only a host-side stand-in, so the address must come from
@@ -79,7 +77,7 @@ int scratch_for_current_device(void **out) {
         return pfac::set_error(PFAC_EINVAL, "pfac_match_noalloc: device %d out of range", dev);
     std::lock_guard<std::mutex> lk(g_mu);
     ScratchAddr &c = g_scratch[dev];
-    void *ctx = current_context();
+    const uint64_t ctx = current_context_id();
     if (!c.ptr || !ctx || c.ctx != ctx) {
         void *p = nullptr;
         e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
@@ -89,7 +87,7 @@ int scratch_for_current_device(void **out) {
                                    cudaGetErrorString(e));
         }
         c.ptr = p;
-        c.ctx = current_context();  // the runtime's context exists now
+        c.ctx = current_context_id();  // the runtime's context exists now
     }
     *out = c.ptr;
     return PFAC_OK;
