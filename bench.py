@@ -40,9 +40,6 @@ sys.path.insert(0, ROOT)
 
 import workloads  # noqa: E402
 
-# (plus the resolver kernel where the plan hands queues over)
-
-
 # dram__bytes_read.sum + dram__bytes_write.sum of one scan launch from ncu
 # captures (summaries under profiles/), per workload and scan plan (the
 # autotuner settles on one of near-equal plans), with the digest of the
@@ -66,6 +63,13 @@ MEASURED_TRAFFIC = {
                          "scan_kernel": 2, "records_per_slice": 32, "resolver": 1})],
 }
 KERNEL_SOURCES = ["kernels_q.cuh", "kernels_r.cuh", "kernels.cuh", "table.h"]
+SCAN_NAMES = {
+    "window": "k_scanw with k_wresolve (compressed-table scan and its resolver)",
+    "dense": "k_scand with k_wresolve (compressed-table scan and its resolver)",
+    "queued": "k_scanq (compressed-table scan: scan pass + emit pass)",
+    "register": "k_scanr (compressed-table scan: scan pass + emit pass)",
+    "serial": "k_scan_dense (transition-table scan: scan pass + emit pass)",
+}
 TUNE_SAMPLE = 128 << 20
 E2E_CHUNK = 32 << 20
 
@@ -86,21 +90,14 @@ def kernel_digest():
     return h.hexdigest()[:16]
 
 
-def spelt_workspace(pfac, table, n_bytes, n_seg, plan):
-    """Workspace of a call with the plan's scan kernel, resolver and records
-    fixed by its options."""
-    return pfac.workspace_bytes(table, n_bytes, n_seg, scan_kernel=plan["scan_kernel"],
-                                resolver=plan["resolver"], records_per_slice=plan["records_per_slice"])
-
-
-def launches_per_step(pfac, table, n_bytes, n_seg, plan, opt):
-    """This library's kernel launches of one match call.  A call that takes the
-    window or dense scan kernel (its workspace then differs from the one of
-    the plan spelt out) clears, scans, resolves and expands, and sums chunk
-    counts beyond 65,536 slices; any other scans, sums, expands and emits,
-    with the resolver and the segment pass where the plan has them."""
-    if pfac.workspace_bytes(table, n_bytes, n_seg, **opt) != spelt_workspace(pfac, table, n_bytes, n_seg, plan):
-        return 4 + (1 if n_bytes > (65536 << 9) else 0)
+def launches_per_step(route, n_bytes, n_seg, plan):
+    """This library's kernel launches of one match call.  One that the window
+    or dense scan kernel takes clears, scans, resolves and expands, and sums
+    chunk counts (the window kernel beyond 65,536 slices, else as it scans);
+    any other scans, sums, expands and emits, with the resolver and the
+    segment pass where the plan has them."""
+    if route in ("window", "dense"):
+        return 4 + (1 if route == "dense" or n_bytes > (65536 << 9) else 0)
     return 4 + (1 if plan["resolver"] == 2 else 0) + (1 if n_seg > 1 else 0)
 
 
@@ -445,15 +442,13 @@ def time_cell(pfac, torch, w, dev, stream, args, user_opt, workload_name, graph_
     emit_avg_ms = sum(emit_ms) / K
     kern_ms = scan_avg_ms + emit_avg_ms
     achieved = alg_bytes / (kern_ms / 1e3) / 1e9
+    route = pfac.kernel(table, S, **user_opt)
     roofline = {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm_peak,
                 "unit": "GB/s", "frac": round(achieved / hbm_peak, 4),
                 "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)",
                 "traffic": args.traffic if (args.traffic is not None and graph_steps) else (
                     measured_traffic(workload_name, plan) if not user_opt else None),
-                "kernel": ("k_scanw or k_scand with k_wresolve (compressed-table scan and its resolver)"
-                           if pfac.workspace_bytes(table, N, S, **user_opt) != spelt_workspace(
-                               pfac, table, N, S, plan) else
-                           "k_scanq or k_scanr (compressed-table scan: scan pass + emit pass)"),
+                "kernel": SCAN_NAMES[route],
                 "alg_bytes_per_launch": alg_bytes,
                 "scan_pass_ms": round(scan_avg_ms, 4), "emit_pass_ms": round(emit_avg_ms, 4)}
     cell = {
@@ -473,8 +468,8 @@ def time_cell(pfac, torch, w, dev, stream, args, user_opt, workload_name, graph_
         "suffix_merge": merged,
         "build_s": {"compressed": round(build_s, 3), "dense": round(dense_build_s, 3)},
         "roofline": roofline,
-        "scan_plan": plan, "autotuned": tune, "cuda_graph": bool(graph is not None),
-        "launches_per_step": launches_per_step(pfac, table, N, S, plan, user_opt),
+        "scan_plan": plan, "scan_kernel_run": route, "autotuned": tune, "cuda_graph": bool(graph is not None),
+        "launches_per_step": launches_per_step(route, N, S, plan),
         "wall_s_timed": round(wall, 4),
         "clocks": clk,
     }
@@ -694,6 +689,7 @@ def run_ours(args):
                        prefix_depth=cell["scan_plan"]["prefix_depth"],
                        variant=args.variant or "default", bitmap_copies=args.copies or "auto",
                        autotuned=cell.pop("autotuned"), scan_plan=cell.pop("scan_plan"),
+                       scan_kernel_run=cell.pop("scan_kernel_run"),
                        cuda_graph=cell.pop("cuda_graph")),
         "p50_ms": cell["p50_ms"], "p99_ms": cell["p99_ms"],
         "matches": cell["matches"], "matched_position_frac": cell["matched_position_frac"],

@@ -273,11 +273,13 @@ int pfac_workspace_bytes(const pfac_table *t, uint64_t n_bytes, uint32_t n_segme
  * pfac_match_plan - the scan configuration a pfac_match call with these
  * options would use (no device work).  Library extension: the paper has no
  * counterpart.  Fields are 0 for the uncompressed layout except smem_bytes.
- * Where the options leave every choice to the library, the table has no tuned
- * choice and its pattern set makes a window filter that pays (a filter over
- * short windows of the text, every S-th position looked up; built with the
- * table), the scan pass runs over that filter; the fields then describe the
- * plan that runs without it.
+ * Where the options leave every choice to the library and the table has no
+ * tuned choice, the window kernel (a filter over short windows of the text,
+ * every S-th position looked up, built with the table where the pattern set
+ * makes one that pays) or, for one segment of 2-bit symbols with a record per
+ * position, the dense scan kernel may take the scan pass in place of the plan:
+ * pfac_match_kernel says so, and the fields then describe the plan that runs
+ * without them.
  */
 typedef struct {
     uint32_t variant;        /* 1 or 2, as pfac_match_opts.variant */
@@ -295,6 +297,21 @@ typedef struct {
                                 resolver kernel does (0: thread-serial) */
 } pfac_plan_info;
 int pfac_match_plan(const pfac_table *t, const pfac_match_opts *opts, pfac_plan_info *out);
+
+/*
+ * pfac_match_kernel - which kernel a pfac_match call over n_segments segments
+ * with these options runs as its scan pass (no device work): one of the
+ * PFAC_KERNEL_ values.  The first three are those of
+ * pfac_match_opts.scan_kernel; the others cannot be asked for there.  Library
+ * extension: the paper has no counterpart.
+ */
+#define PFAC_KERNEL_QUEUED 1
+#define PFAC_KERNEL_REGISTER 2
+#define PFAC_KERNEL_SERIAL 3
+#define PFAC_KERNEL_WINDOW 4
+#define PFAC_KERNEL_DENSE 5
+int pfac_match_kernel(const pfac_table *t, uint32_t n_segments, const pfac_match_opts *opts,
+                      uint32_t *kernel);
 
 /*
  * pfac_match_async - match a device-resident text (Section 2.3), fully

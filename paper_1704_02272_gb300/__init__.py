@@ -6,7 +6,7 @@ builder of the bitmap trie and hand-written sm_103a kernels.  This package is
 its thin Python binding; importing it fails when the library is not built.
 """
 from .binding import (ID_BITS, LAYOUT_COMPRESSED, LAYOUT_DENSE, VARIANT_DEFAULT,  # noqa: F401
-                      VARIANT_DSMEM, VARIANT_FILTER, PfacError, Server, Table, autotune,
+                      VARIANT_DSMEM, VARIANT_FILTER, PfacError, Server, Table, autotune, kernel,
                       match, match_async, match_host, match_into, match_noalloc, plan, single_segment, unpack, verify,
                       verify_into,
                       version,

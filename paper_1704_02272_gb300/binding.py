@@ -123,6 +123,8 @@ def _load():
                                          ctypes.POINTER(u64)]
     lib.pfac_match_plan.restype = ctypes.c_int
     lib.pfac_match_plan.argtypes = [vp, ctypes.POINTER(MatchOpts), ctypes.POINTER(PlanInfo)]
+    lib.pfac_match_kernel.restype = ctypes.c_int
+    lib.pfac_match_kernel.argtypes = [vp, u32, ctypes.POINTER(MatchOpts), ctypes.POINTER(u32)]
     lib.pfac_match_host.restype = ctypes.c_int
     lib.pfac_match_host.argtypes = [vp, vp, u64, vp, u32, vp, u64, ctypes.POINTER(u64), u64,
                                     ctypes.POINTER(MatchOpts), vp]
@@ -316,6 +318,17 @@ def plan(table: Table, **opt) -> dict:
     r = PlanInfo()
     _check(LIB.pfac_match_plan(table.handle, ctypes.byref(o), ctypes.byref(r)))
     return {f: getattr(r, f) for f, _ in PlanInfo._fields_ if f != "reserved"}
+
+
+KERNEL_NAMES = {1: "queued", 2: "register", 3: "serial", 4: "window", 5: "dense"}
+
+
+def kernel(table: Table, n_segments: int = 1, **opt) -> str:
+    """pfac_match_kernel: the kernel that a match over n_segments segments with
+    these options runs as its scan pass."""
+    o, k = _opts(**opt), ctypes.c_uint32()
+    _check(LIB.pfac_match_kernel(table.handle, n_segments, ctypes.byref(o), ctypes.byref(k)))
+    return KERNEL_NAMES[k.value]
 
 
 def match_host(table: Table, text: torch.Tensor, seg: torch.Tensor, out: torch.Tensor,

@@ -400,7 +400,7 @@ struct Plan {
     void *kernel_d;
 };
 
-enum { SCAN_QUEUED = 1, SCAN_REGISTER = 2, SCAN_SERIAL = 3 };
+enum { SCAN_QUEUED = PFAC_KERNEL_QUEUED, SCAN_REGISTER = PFAC_KERNEL_REGISTER, SCAN_SERIAL = PFAC_KERNEL_SERIAL };
 
 struct WsLayout {
     uint64_t hdr, tile_m, tile_k, key_off, chunk, ovf, recs, bounds, defer, dbatch, total;
@@ -1114,6 +1114,17 @@ extern "C" int pfac_match_plan(const pfac_table *t, const pfac_match_opts *opts,
     out->scan_kernel = (uint32_t)pl.kind;
     out->records_per_slice = pl.unit_cap;
     out->resolver = pl.kind == SCAN_SERIAL ? 0u : (pl.defer ? 2u : 1u);
+    return PFAC_OK;
+}
+
+extern "C" int pfac_match_kernel(const pfac_table *t, uint32_t n_segments,
+                                 const pfac_match_opts *opts, uint32_t *kernel) {
+    clear_error();
+    if (!t || !kernel) return set_error(PFAC_EINVAL, "pfac_match_kernel: NULL argument");
+    Plan pl;
+    const int rc = make_plan(t, n_segments, opts, &pl);
+    if (rc) return rc;
+    *kernel = pl.win ? PFAC_KERNEL_WINDOW : pl.dsc ? PFAC_KERNEL_DENSE : (uint32_t)pl.kind;
     return PFAC_OK;
 }
 
