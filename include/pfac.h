@@ -422,19 +422,23 @@ void pfac_match_host_release(void);
  * fail with out-of-memory halfway through a stream, or in a process whose
  * device-memory budget is fixed at start-up.  This call allocates nothing:
  * no cudaMalloc, no cudaFree, no allocating library routine.  Its scratch is
- * a device array of PFAC_NOALLOC_SCRATCH_BYTES compiled into the library,
- * which every GPU that loads the library holds until the process exits.
+ * a device array of PFAC_NOALLOC_SCRATCH_BYTES (and 32 KiB for what does not
+ * grow with the input) compiled into the library, which every GPU that loads
+ * the library holds until the process exits.
  *
  * Arguments are those of pfac_match_async without the workspace.  The
  * caller still provides the input, the offsets, the output keys, d_count and
  * (optionally) d_status.
  *
  * Limits and rules:
- *   - the scratch an input needs grows with its size (about 0.55 bytes per
- *     input byte, pfac_workspace_bytes gives the exact figure); where the
- *     library's own choices (512 records per slice, the resolver kernel's
- *     buffer) would not fit, the call takes 32 records per slice and the scan
- *     kernel's own resolution instead (unless the caller set both); inputs
+ *   - the scratch an input needs grows with its size (0.55 to 0.85 bytes per
+ *     input byte with 32 records per slice, 8.3 with 512;
+ *     pfac_workspace_bytes gives the exact figure); where the library's own
+ *     choices (512 records per slice, the buffer of the window kernel's
+ *     entries or of the resolver kernel's queues) would not fit, from about
+ *     40 MiB of input on, the call takes 32 records per slice and the queued
+ *     or register-staged kernel's own resolution instead (unless the caller
+ *     set both), which is slower; inputs
  *     that need more than PFAC_NOALLOC_SCRATCH_BYTES even so (roughly 58 MiB
  *     of input) are rejected with PFAC_EINVAL and a message naming both
  *     sizes, before any device work;

@@ -46,6 +46,21 @@ void clear_error();
 // with another GPU's pointers.
 int check_table_device(const pfac_table *t, void *cuda_stream, const char *who);
 
+// Bytes of a workspace that do not grow with the input, at most: a fixed
+// scratch or pool of N bytes is made this much larger, so that it holds what
+// takes N bytes for its input alone.
+constexpr uint64_t WS_FIXED_BYTES = 32 << 10;
+
+// The options that need the least scratch: the library's choice of the rest,
+// 32 records a slice, and no buffer for a resolver launch.
+inline pfac_match_opts lean_opts(const pfac_match_opts *opts) {
+    pfac_match_opts o{};
+    if (opts) o = *opts;
+    if (!o.records_per_slice) o.records_per_slice = 32;
+    if (!o.resolver) o.resolver = 1;
+    return o;
+}
+
 // Stream-ordered scratch from the library's own pool of the current context
 // (freed with cudaFreeAsync), and giving back what the pool keeps (waits for
 // the device first; nothing where there is no pool).

@@ -1081,14 +1081,22 @@ extern "C" int pfac_workspace_bytes(const pfac_table *t, uint64_t n_bytes, uint3
     Plan pl;
     const int rc = make_plan(t, n_segments, opts, &pl);
     if (rc) return rc;
-    *bytes = ws_layout(n_bytes, n_segments, pl).total;
-    if (pl.unit_cap == (uint32_t)SLICE && n_segments > 1) {
-        // enough for fewer segments too (a chunk of a longer text), where
-        // another kernel may take the call
-        Plan one;
-        if (make_plan(t, 1, opts, &one) == PFAC_OK)
-            *bytes = std::max(*bytes, ws_layout(n_bytes, 1, one).total);
-    }
+    // enough too for the same call with options that choose its scan (the plan
+    // without the window or dense kernel), and for fewer segments (a chunk of
+    // a longer text), where another kernel may take it
+    auto total = [&](uint32_t n_seg, Plan &p) {
+        uint64_t b = ws_layout(n_bytes, n_seg, p).total;
+        if (p.win || p.dsc) {
+            p.win = p.dsc = false;
+            b = std::max(b, ws_layout(n_bytes, n_seg, p).total);
+        }
+        return b;
+    };
+    const bool full = pl.unit_cap == (uint32_t)SLICE;
+    *bytes = total(n_segments, pl);
+    Plan one;
+    if (full && n_segments > 1 && make_plan(t, 1, opts, &one) == PFAC_OK)
+        *bytes = std::max(*bytes, total(1, one));
     return PFAC_OK;
 }
 

@@ -10,8 +10,8 @@
 // no cudaMalloc, no cudaFree and no call into an allocating library: the
 // scratch (per-tile counters, match records and segment lists) lives in
 // `g_noalloc_scratch` below, a file-scope device array of
-// PFAC_NOALLOC_SCRATCH_BYTES that every GPU which loads this library holds
-// until the process exits.
+// PFAC_NOALLOC_SCRATCH_BYTES and a little that every GPU which loads this
+// library holds until the process exits.
 #include <cuda_runtime.h>
 #include <string.h>
 
@@ -19,7 +19,8 @@
 
 #include "internal.h"
 
-static __device__ __align__(256) uint8_t g_noalloc_scratch[PFAC_NOALLOC_SCRATCH_BYTES];
+static __device__ __align__(256) uint8_t
+    g_noalloc_scratch[PFAC_NOALLOC_SCRATCH_BYTES + pfac::WS_FIXED_BYTES];
 
 namespace {
 
@@ -110,31 +111,28 @@ extern "C" int pfac_match_noalloc(const pfac_table *t, const uint8_t *d_input, u
     rc = pfac_workspace_bytes(t, n_bytes, n_segments, opts, &need);
     if (rc) return rc;
     // library choices that take more scratch (a record per position, 8 bytes
-    // per input byte; the resolver kernel's buffer) give way to the smaller
-    // record space and the scan's own resolution when only those fit
+    // per input byte; the window kernel's or the resolver's buffer) give way
+    // to the smaller record space and the scan's own resolution when only
+    // those fit
+    constexpr uint64_t room = sizeof g_noalloc_scratch;
     pfac_match_opts o32;
-    if (need > (uint64_t)PFAC_NOALLOC_SCRATCH_BYTES &&
-        !(opts && opts->records_per_slice && opts->resolver)) {
-        if (opts) o32 = *opts;
-        else memset(&o32, 0, sizeof o32);
-        if (!o32.records_per_slice) o32.records_per_slice = 32;
-        if (!o32.resolver) o32.resolver = 1;
+    if (need > room && !(opts && opts->records_per_slice && opts->resolver)) {
+        o32 = pfac::lean_opts(opts);
         uint64_t need32 = 0;
-        if (pfac_workspace_bytes(t, n_bytes, n_segments, &o32, &need32) == PFAC_OK &&
-            need32 <= (uint64_t)PFAC_NOALLOC_SCRATCH_BYTES) {
+        if (pfac_workspace_bytes(t, n_bytes, n_segments, &o32, &need32) == PFAC_OK && need32 <= room) {
             opts = &o32;
             need = need32;
         }
         pfac::clear_error();
     }
-    if (need > (uint64_t)PFAC_NOALLOC_SCRATCH_BYTES)
+    if (need > room)
         return pfac::set_error(PFAC_EINVAL,
                                "pfac_match_noalloc: an input of %llu bytes in %u segments needs "
                                "%llu bytes of scratch, more than the built-in %llu; split the "
                                "input or use pfac_match_async with a workspace",
                                (unsigned long long)n_bytes, n_segments,
                                (unsigned long long)need,
-                               (unsigned long long)PFAC_NOALLOC_SCRATCH_BYTES);
+                               (unsigned long long)room);
     void *scratch = nullptr;
     rc = scratch_for_current_device(&scratch);
     if (rc) return rc;

@@ -95,6 +95,11 @@ struct Request {
     uint64_t n;
     const uint64_t *h_seg;
     uint32_t nseg;
+    // matched with the options that need the least scratch, where the
+    // library's choice does not fit the pool
+    bool lean = false;
+    pfac_match_opts lean_o{};
+    const pfac_match_opts *opts() const { return lean ? &lean_o : nullptr; }
     double t_submit = 0, t_admit = 0, t_done = 0, t_issued = 0, t_counted = 0;
     int status = PFAC_OK;
     std::vector<uint64_t> keys;  // keys outside the arena
@@ -147,9 +152,9 @@ namespace {
 // Bytes of one request's device block: input, offsets, workspace, count and
 // status, output keys.
 uint64_t request_bytes(const pfac_table *t, uint64_t n, uint32_t nseg, uint64_t cap,
-                       uint64_t *ws_out) {
+                       const pfac_match_opts *opts, uint64_t *ws_out) {
     uint64_t ws = 0;
-    if (pfac_workspace_bytes(t, n, nseg, nullptr, &ws) != PFAC_OK) return 0;
+    if (pfac_workspace_bytes(t, n, nseg, opts, &ws) != PFAC_OK) return 0;
     *ws_out = ws;
     auto a = [](uint64_t x) { return (x + 255) & ~255ull; };
     return a(n) + a(8ull * (nseg + 1)) + a(ws) + 256 + a(8 * cap);
@@ -162,7 +167,7 @@ uint64_t first_capacity(uint64_t n) { return n / 8 > 4096 ? n / 8 : 4096; }
 bool admit(pfac_server *s, Slot &sl, Request *r) {
     const uint64_t cap = first_capacity(r->n);
     uint64_t ws = 0;
-    const uint64_t need = request_bytes(s->t, r->n, r->nseg, cap, &ws);
+    const uint64_t need = request_bytes(s->t, r->n, r->nseg, cap, r->opts(), &ws);
     uint64_t off = 0;
     if (!need || !s->pool.alloc(need, &off)) return false;
     auto a = [](uint64_t x) { return (x + 255) & ~255ull; };
@@ -187,7 +192,7 @@ bool admit(pfac_server *s, Slot &sl, Request *r) {
     int rc = e == cudaSuccess ? PFAC_OK : PFAC_ECUDA;
     if (rc == PFAC_OK)
         rc = pfac_match_async(s->t, d_in, r->n, d_seg, r->nseg, d_out, cap, d_small,
-                              (int32_t *)(d_small + 1), d_ws, ws, nullptr, sl.stream);
+                              (int32_t *)(d_small + 1), d_ws, ws, r->opts(), sl.stream);
     if (rc == PFAC_OK)
         e = cudaMemcpyAsync(sl.h_small, d_small, 16, cudaMemcpyDeviceToHost, sl.stream);
     if (rc == PFAC_OK && e == cudaSuccess) e = cudaEventRecord(sl.ev, sl.stream);
@@ -232,7 +237,7 @@ Block block_of(pfac_server *s, const Slot &sl, const Request *r) {
     b.in = s->pool.base + sl.off;
     b.seg = (uint64_t *)(b.in + a(r->n));
     b.ws_bytes = 0;
-    pfac_workspace_bytes(s->t, r->n, r->nseg, nullptr, &b.ws_bytes);
+    pfac_workspace_bytes(s->t, r->n, r->nseg, r->opts(), &b.ws_bytes);
     b.ws = (uint8_t *)b.seg + a(8ull * (r->nseg + 1));
     b.small = (uint64_t *)(b.ws + a(b.ws_bytes));
     return b;
@@ -281,7 +286,7 @@ bool rematch(pfac_server *s, Slot &sl, Request *r, uint64_t cnt, uint64_t *dst) 
         return false;
     }
     const int rc = pfac_match_async(s->t, b.in, r->n, b.seg, r->nseg, sl.d_big, cnt, b.small,
-                                    (int32_t *)(b.small + 1), b.ws, b.ws_bytes, nullptr, sl.stream);
+                                    (int32_t *)(b.small + 1), b.ws, b.ws_bytes, r->opts(), sl.stream);
     cudaError_t e = cudaSuccess;
     if (rc == PFAC_OK)
         e = cudaMemcpyAsync(sl.h_small, b.small, 16, cudaMemcpyDeviceToHost, sl.stream);
@@ -397,12 +402,13 @@ extern "C" int pfac_server_create(const pfac_table *t, const pfac_server_opts *o
     pfac_server_opts opt{};
     if (o) opt = *o;
     const uint32_t n_slots = opt.n_slots ? opt.n_slots : 4;
-    const uint64_t pool = opt.device_bytes ? opt.device_bytes : (1ull << 30);
+    const uint64_t bytes = opt.device_bytes ? opt.device_bytes : (1ull << 30);
+    const uint64_t pool = bytes + WS_FIXED_BYTES;
     pfac_server *s = new (std::nothrow) pfac_server();
     if (!s) return set_error(PFAC_ENOMEM, "pfac_server_create: host allocation");
     cudaGetDevice(&s->device);
     s->t = t;
-    s->max_req = opt.max_request_bytes ? opt.max_request_bytes : pool / 4;
+    s->max_req = opt.max_request_bytes ? opt.max_request_bytes : bytes / 4;
     cudaError_t e = cudaMalloc((void **)&s->d_pool, pool);
     if (e != cudaSuccess) {
         delete s;
@@ -447,7 +453,11 @@ extern "C" int pfac_server_submit(pfac_server *s, const uint8_t *h_input, uint64
     if (n_bytes && n_segments == 0)
         return set_error(PFAC_EINVAL, "pfac_server_submit: a non-empty input needs a segment");
     uint64_t ws = 0;
-    const uint64_t need = request_bytes(s->t, n_bytes, n_segments, first_capacity(n_bytes), &ws);
+    const uint64_t cap = first_capacity(n_bytes);
+    uint64_t need = request_bytes(s->t, n_bytes, n_segments, cap, nullptr, &ws);
+    const pfac_match_opts lean = lean_opts(nullptr);
+    const bool use_lean = need > s->pool.size;
+    if (use_lean) need = request_bytes(s->t, n_bytes, n_segments, cap, &lean, &ws);
     if (n_bytes > s->max_req || need > s->pool.size)
         return set_error(PFAC_ENOMEM, "pfac_server_submit: request of %llu bytes exceeds the "
                          "server's limits", (unsigned long long)n_bytes);
@@ -457,6 +467,8 @@ extern "C" int pfac_server_submit(pfac_server *s, const uint8_t *h_input, uint64
     r->n = n_bytes;
     r->h_seg = h_seg_offsets;
     r->nseg = n_segments;
+    r->lean = use_lean;
+    r->lean_o = lean;
     r->t_submit = now_s();
     {
         std::lock_guard<std::mutex> lk(s->mu);
