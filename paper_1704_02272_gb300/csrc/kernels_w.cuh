@@ -141,27 +141,46 @@ __device__ __forceinline__ uint32_t w_filter(const uint32_t (&w)[9], const WCons
 
 // One match: a record in the slice's space while it has room (in any order),
 // and the slice's counts: records above bit UNIT_KEY_BITS of its word, keys
-// below, so that one atomic takes the slots and counts the keys.  (A slice
-// with more matches than its space is walked again by the expansion.)  The
-// calling lanes' matches of a slice share one atomic: where most starts match,
-// a warp's 32 lie in one or two slices and queued on its word (8 MiB of one
-// symbol that two patterns repeat: 1,602 -> 655 us a call).  With few slices
-// the chunks' key counts are added up here too; with many, neighbouring
+// below, so that one atomic takes the slot and counts the keys.  (A slice with
+// more matches than its space is walked again by the expansion.)  With few
+// slices the chunks' key counts are added up here too; with many, neighbouring
 // matches would queue on one chunk's word (1 GiB of packets: 0.8 instead of
 // 0.36 ms), and k_reduce sums them.
+//
+// SHARED: calling lanes whose matches lie in one slice add once.  For the
+// scan's own walks, where most starts may match: 32 adds then queued on one
+// word (8 MiB of one symbol that two patterns repeat, all / shared: 1,079 /
+// 610 us a call).  Not for the resolver, whose few matches lie apart: shared
+// there too, 1 GiB of packets 1,204 -> 1,222 us, and by slices told apart with
+// a match instruction 1,249.
+template <bool SHARED>
 __device__ __forceinline__ void w_emit(const MatchParams &P, uint32_t u, uint32_t pos, uint32_t fin) {
     u = (uint32_t)chk(P, u, P.n_tiles);
-    const uint32_t cap = P.unit_cap, lane = threadIdx.x & 31;
-    const uint32_t same = __match_any_sync(__activemask(), u), first = __ffs(same) - 1;
-    // (lists of at most 2^24 ids: a warp's fit 32 bits)
-    const uint32_t keys = __reduce_add_sync(same, (uint32_t)fin_len_c(P, fin));
-    uint32_t rank = 0;
-    if (lane == first) {
-        rank = (uint32_t)(atomicAdd((unsigned long long *)(P.tile_k + u),
-                                    ((unsigned long long)__popc(same) << UNIT_KEY_BITS) | keys) >> UNIT_KEY_BITS);
-        if (P.chunk_adds) atomicAdd((unsigned long long *)(P.chunk + (u >> P.chunk_shift)), (unsigned long long)keys);
+    const uint32_t cap = P.unit_cap;
+    unsigned long long keys = fin_len_c(P, fin);
+    uint32_t n = 1, lower = 0;  // matches of this add, and those before the lane's
+    uint32_t act = 0, first = 0;
+    bool one = false, adds = true;
+    if (SHARED) {
+        act = __activemask();
+        first = __ffs(act) - 1;
+        one = __all_sync(act, u == __shfl_sync(act, u, first));
+        if (one) {
+            // (lists of at most 2^24 ids: a warp's fit 32 bits)
+            keys = __reduce_add_sync(act, (uint32_t)keys);
+            n = __popc(act);
+            const uint32_t lane = threadIdx.x & 31;
+            lower = __popc(act & ((1u << lane) - 1u));
+            adds = lane == first;
+        }
     }
-    rank = __shfl_sync(same, rank, first) + __popc(same & ((1u << lane) - 1u));
+    uint32_t rank = 0;
+    if (adds) {
+        rank = (uint32_t)(atomicAdd((unsigned long long *)(P.tile_k + u),
+                                    ((unsigned long long)n << UNIT_KEY_BITS) | keys) >> UNIT_KEY_BITS);
+        if (P.chunk_adds) atomicAdd((unsigned long long *)(P.chunk + (u >> P.chunk_shift)), keys);
+    }
+    if (SHARED && one) rank = __shfl_sync(act, rank, first) + lower;
     if (rank < cap) P.recs[(size_t)u * cap + rank] = ((uint64_t)pos << 32) | fin;
 }
 
@@ -227,7 +246,7 @@ static __device__ __noinline__ void w_walk(const MatchParams *PP, uint64_t p) {
     const MatchParams &P = *PP;
     const uint32_t u = (uint32_t)(p >> SLICE_SHIFT), pos = (uint32_t)p & (SLICE - 1);
     const uint32_t fin = w_walk_any(P, (uint64_t)u << SLICE_SHIFT, pos, w_limit<false>(P, u, p));
-    if (fin) w_emit(P, u, pos, fin);
+    if (fin) w_emit<true>(P, u, pos, fin);
 }
 
 // The text around a start, loaded without branches so that several starts'
@@ -560,7 +579,7 @@ template <int DENSE>
 __device__ __forceinline__ void w_result(const MatchParams &P, uint32_t u, uint32_t pos, uint32_t slot,
                                          uint32_t fin) {
     if (!DENSE) {
-        if (fin) w_emit(P, u, pos, fin);
+        if (fin) w_emit<false>(P, u, pos, fin);
         return;
     }
     P.recs[(size_t)u * P.unit_cap + slot] = ((uint64_t)pos << 32) | fin;
