@@ -464,12 +464,14 @@ int pfac_match_noalloc(const pfac_table *t, const uint8_t *d_input, uint64_t n_b
  * (the prefix depth resolved in shared memory, whether the prefix entries
  * live in shared memory, the child masks, the gram filter or the prefix
  * bitmap as the first stage, and how many copies of that bitmap are spread
- * over the shared-memory banks).  Each candidate runs the scan kernel
- * on the caller's device-resident sample (same argument rules as
- * pfac_match_async); the fastest becomes the table's default for later
- * pfac_match calls without options.  With a non-NULL cache_path the choice
- * is read from / appended to that text file, keyed by alphabet size,
- * pattern count, maximum pattern length, sample size class and GPU name.
+ * over the shared-memory banks).  Each candidate, the library's own choice
+ * among them, runs whole calls on the caller's device-resident sample (same
+ * argument rules as pfac_match_async); the fastest becomes the table's default
+ * for later pfac_match calls without options.  With a non-NULL cache_path the
+ * choice (also the library's own) is read from / appended to that text file,
+ * keyed by alphabet size, pattern count, maximum pattern length, sample size
+ * class and GPU name.  A cached choice is applied as it stands: after an
+ * update of the library, a new file has the candidates compared again.
  * Synchronous (waits for the stream).  out may be NULL.
  */
 typedef struct {

@@ -1,11 +1,11 @@
 // Autotuner of the scan configuration (pfac_autotune).  For a built table
-// and a device-resident sample it times the scan kernel for each candidate
-// (the scan kernel: queued or register-staged x prefix depth resolved in
-// shared memory x entries in shared memory or not x child masks on or off x
-// the first stage (prefix bitmap, gram filter or prefix bytes) x copies of
-// that bitmap over the banks x CTA width), keeps the fastest as the
-// table's default, and can remember the choice in a small text cache keyed by
-// the table's shape and the GPU.
+// and a device-resident sample it times a call with each candidate (the scan
+// kernel: queued or register-staged x prefix depth resolved in shared memory x
+// entries in shared memory or not x child masks on or off x the first stage
+// (prefix bitmap, gram filter or prefix bytes) x copies of that bitmap over
+// the banks x CTA width) and with the library's own choice, keeps the fastest
+// as the table's default, and can remember the choice in a small text cache
+// keyed by the table's shape and the GPU.
 #include <cuda_runtime.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -13,6 +13,7 @@
 
 #include <algorithm>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "internal.h"
@@ -42,6 +43,7 @@ std::string cache_key(const pfac_table *t, uint64_t n_bytes, uint32_t n_segments
 
 // A cache line: key, variant, depth, copies, masks, gram filter, prefix
 // bytes, warps per CTA, scan kernel, records per slice, resolver, time.
+// A line of zeros says that the library's own choice was the fastest.
 // Lines without the scan kernel (written before the register-staged kernel
 // existed) name the queued one; lines without the records or the resolver
 // leave them to the library.
@@ -91,6 +93,12 @@ bool cache_lookup(const char *path, const std::string &key, uint32_t *v, uint32_
     return found;
 }
 
+// A cached choice that fixes nothing: the library's own.
+template <class... U>
+bool own_choice(U... fields) {
+    return ((fields == 0) && ...);
+}
+
 }  // namespace
 
 extern "C" int pfac_autotune(pfac_table *t, const uint8_t *d_sample, uint64_t n_bytes,
@@ -106,8 +114,9 @@ extern "C" int pfac_autotune(pfac_table *t, const uint8_t *d_sample, uint64_t n_
         float ms;
         if (cache_lookup(cache_path, key, &v, &k, &c, &mk, &gf, &pb, &nw, &kind, &rp, &rsv, &ms) &&
             rsv <= 2 &&
-            k >= t->kmin && k <= t->kmax && (gf != 2 || t->dev.g_len) &&
-            (pb != 2 || t->dev.B[k])) {
+            (own_choice(v, k, c, mk, gf, pb, nw, kind, rp, rsv) ||
+             (k >= t->kmin && k <= t->kmax && (gf != 2 || t->dev.g_len) &&
+              (pb != 2 || t->dev.B[k])))) {
             t->tuned_bytes = pb;
             t->tuned_nw = nw;
             t->tuned_kernel = kind;
@@ -133,10 +142,11 @@ extern "C" int pfac_autotune(pfac_table *t, const uint8_t *d_sample, uint64_t n_
             // a cached choice that no longer makes a plan (an edited or
             // foreign cache line) is dropped and the table tuned afresh
             pfac_plan_info pi;
-            const bool sane = (kind == 1 || kind == 2) && (nw == 0 || nw == 16 || nw == 24) &&
-                              (rp == 0 || rp == 32 || rp == 512) &&
-                              v <= 2 && mk <= 2 && gf <= 2 && pb <= 2 && c <= 32 &&
-                              (c & (c - 1)) == 0;
+            const bool sane = own_choice(v, k, c, mk, gf, pb, nw, kind, rp, rsv) ||
+                              ((kind == 1 || kind == 2) && (nw == 0 || nw == 16 || nw == 24) &&
+                               (rp == 0 || rp == 32 || rp == 512) &&
+                               v <= 2 && mk <= 2 && gf <= 2 && pb <= 2 && c <= 32 &&
+                               (c & (c - 1)) == 0);
             if (sane && pfac_match_plan(t, nullptr, &pi) == PFAC_OK) {
                 if (out) *out = res;
                 return PFAC_OK;
@@ -161,7 +171,8 @@ extern "C" int pfac_autotune(pfac_table *t, const uint8_t *d_sample, uint64_t n_
 
     struct Cand {
         uint32_t var, k, copies, masks, gram, bytes, nw, kernel;
-        float ms;
+        float ms;          // its scan kernel's launches
+        float call = 0.f;  // the whole call, which candidates are compared by
         uint32_t recs = 0;  // records per slice (0: the library's choice)
         uint32_t resolver = 0;  // who resolves the queues (0: the library's choice)
     };
@@ -219,25 +230,23 @@ extern "C" int pfac_autotune(pfac_table *t, const uint8_t *d_sample, uint64_t n_
     void *ws = nullptr, *small = nullptr;
     cudaError_t e = cudaMalloc(&ws, ws_max ? ws_max : 256);
     if (e == cudaSuccess) e = cudaMalloc(&small, 256);
-    cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr, e3 = nullptr;
-    if (e == cudaSuccess) e = cudaEventCreate(&e0);
-    if (e == cudaSuccess) e = cudaEventCreate(&e1);
-    if (e == cudaSuccess) e = cudaEventCreate(&e2);
-    if (e == cudaSuccess) e = cudaEventCreate(&e3);
+    cudaEvent_t ev[6] = {};  // around the scan, the emit launch and the call
+    for (cudaEvent_t &v : ev)
+        if (e == cudaSuccess) e = cudaEventCreate(&v);
     if (e != cudaSuccess) {
         cudaFree(ws);
         cudaFree(small);
-        if (e0) cudaEventDestroy(e0);
-        if (e1) cudaEventDestroy(e1);
-        if (e2) cudaEventDestroy(e2);
+        for (cudaEvent_t v : ev)
+            if (v) cudaEventDestroy(v);
         cudaGetLastError();
         return set_error(PFAC_ENOMEM, "pfac_autotune: %s", cudaGetErrorString(e));
     }
     uint64_t *d_cnt = (uint64_t *)small;
     int32_t *d_st = (int32_t *)((uint8_t *)small + 128);
-    // the scan kernel's time for one candidate (both launches: the scan pass
-    // and the emit pass), median of three after a warm-up; false when it
-    // does not run
+    // one candidate's time, median of three after a warm-up; false when it
+    // does not run.  Whole calls are compared: the kernels share a call's work
+    // out differently (who finds the segments, who walks full slices again),
+    // so that parts of it do not compare.
     auto time_cand = [&](Cand &c) -> bool {
         pfac_match_opts o = opts_of(c);
         uint64_t b = 0;
@@ -248,26 +257,31 @@ extern "C" int pfac_autotune(pfac_table *t, const uint8_t *d_sample, uint64_t n_
             clear_error();
             return false;
         }
-        o.ev_scan_begin = e0;
-        o.ev_scan_end = e1;
-        o.ev_emit_begin = e2;
-        o.ev_emit_end = e3;
-        float t3[3];
+        o.ev_scan_begin = ev[0];
+        o.ev_scan_end = ev[1];
+        o.ev_emit_begin = ev[2];
+        o.ev_emit_end = ev[3];
+        std::pair<float, float> t3[3];  // call, scan
         for (int r = 0; r < 3; r++) {
-            rc = pfac_match_async(t, d_sample, n_bytes, d_seg_offsets, n_segments, nullptr, 0,
-                                  d_cnt, d_st, ws, b, &o, st);
-            float ms_scan = 0.f, ms_emit = 0.f;
-            if (rc == PFAC_OK && cudaEventSynchronize(e3) == cudaSuccess &&
-                cudaEventElapsedTime(&ms_scan, e0, e1) == cudaSuccess &&
-                cudaEventElapsedTime(&ms_emit, e2, e3) == cudaSuccess) {
-                t3[r] = ms_scan + ms_emit;
+            rc = cudaEventRecord(ev[4], st) == cudaSuccess ? PFAC_OK : PFAC_ECUDA;
+            if (rc == PFAC_OK)
+                rc = pfac_match_async(t, d_sample, n_bytes, d_seg_offsets, n_segments, nullptr, 0,
+                                      d_cnt, d_st, ws, b, &o, st);
+            float ms_call = 0.f, ms_scan = 0.f, ms_emit = 0.f;
+            if (rc == PFAC_OK && cudaEventRecord(ev[5], st) == cudaSuccess &&
+                cudaEventSynchronize(ev[5]) == cudaSuccess &&
+                cudaEventElapsedTime(&ms_call, ev[4], ev[5]) == cudaSuccess &&
+                cudaEventElapsedTime(&ms_scan, ev[0], ev[1]) == cudaSuccess &&
+                cudaEventElapsedTime(&ms_emit, ev[2], ev[3]) == cudaSuccess) {
+                t3[r] = {ms_call, ms_scan + ms_emit};
             } else {
                 clear_error();
                 return false;
             }
         }
         std::sort(t3, t3 + 3);
-        c.ms = t3[1];
+        c.call = t3[1].first;
+        c.ms = t3[1].second;
         return true;
     };
     std::vector<Cand> timed;
@@ -277,7 +291,7 @@ extern "C" int pfac_autotune(pfac_table *t, const uint8_t *d_sample, uint64_t n_
     if (!timed.empty()) {
         Cand best0 = timed[0];
         for (const Cand &c : timed)
-            if (c.var && c.ms < best0.ms) best0 = c;
+            if (c.var && c.call < best0.call) best0 = c;
         pfac_plan_info pi;
         pfac_match_opts o = opts_of(best0);
         if (best0.var && pfac_match_plan(t, &o, &pi) == PFAC_OK) {
@@ -289,7 +303,7 @@ extern "C" int pfac_autotune(pfac_table *t, const uint8_t *d_sample, uint64_t n_
         // the best of those with the other resolution of the queues
         Cand best1 = best0;
         for (const Cand &c : timed)
-            if (c.var && c.ms < best1.ms) best1 = c;
+            if (c.var && c.call < best1.call) best1 = c;
         o = opts_of(best1);
         if (best1.var && pfac_match_plan(t, &o, &pi) == PFAC_OK && pi.resolver) {
             Cand alt = best1;
@@ -301,10 +315,7 @@ extern "C" int pfac_autotune(pfac_table *t, const uint8_t *d_sample, uint64_t n_
     int32_t h_st = 0;
     e = cudaMemcpyAsync(&h_st, d_st, 4, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    cudaEventDestroy(e2);
-    cudaEventDestroy(e3);
+    for (cudaEvent_t v : ev) cudaEventDestroy(v);
     cudaFree(ws);
     cudaFree(small);
     if (e != cudaSuccess) return set_error(PFAC_ECUDA, "pfac_autotune: %s", cudaGetErrorString(e));
@@ -313,7 +324,7 @@ extern "C" int pfac_autotune(pfac_table *t, const uint8_t *d_sample, uint64_t n_
     const Cand &def = timed[0];
     Cand best = def;
     for (const Cand &c : timed)
-        if (c.var && c.ms < best.ms) best = c;
+        if (c.var && c.call < best.call) best = c;
     res.default_ms = def.var == 0 ? def.ms : 0.f;
     res.n_tried = (uint32_t)timed.size();
     if (best.var) {
@@ -339,7 +350,7 @@ extern "C" int pfac_autotune(pfac_table *t, const uint8_t *d_sample, uint64_t n_
     res.records_per_slice = best.recs;
     res.resolver = best.resolver;
     res.scan_ms = best.ms;
-    if (cache_path && best.var) {
+    if (cache_path) {
         FILE *f = fopen(cache_path, "a");
         if (f) {
             fprintf(f, "%s %u %u %u %u %u %u %u %u %u %u %.6f\n", key.c_str(), best.var, best.k,
