@@ -147,7 +147,9 @@ constexpr int UNIT_KEY_BITS = 40;
 // input index through chk(), which, for an index at or past its bound,
 // records ST_DEVICE in the call's status word (the call then reports
 // PFAC_EDEVICE) and returns 0, always a valid index, so that no access leaves
-// its array.  In the regular build chk() is the index itself.
+// its array.  In the regular build chk() is the index itself.  Left out are
+// indices that the line before has compared with their bound, and the loops
+// that fill shared memory, which run to its size.
 #ifdef PFAC_CHECKED
 constexpr bool CHECKED = true;
 __device__ __forceinline__ uint64_t chk(const MatchParams &P, uint64_t i, uint64_t n) {
@@ -159,6 +161,16 @@ __device__ __forceinline__ uint64_t chk(const MatchParams &P, uint64_t i, uint64
 constexpr bool CHECKED = false;
 __device__ __forceinline__ uint64_t chk(const MatchParams &, uint64_t i, uint64_t) { return i; }
 #endif
+
+// The same for a 32-bit index, and for `len` bytes of the input.
+__device__ __forceinline__ uint32_t chk32(const MatchParams &P, uint32_t i, uint64_t n) {
+    return CHECKED ? (uint32_t)chk(P, i, n) : i;
+}
+__device__ __forceinline__ const uint8_t *chk_in(const MatchParams &P, const uint8_t *p, uint64_t len) {
+    if (!CHECKED) return p;
+    const uint64_t i = (uint64_t)(p - P.in);
+    return P.in + (i + len > P.n ? chk(P, 1, 0) : i);
+}
 
 // ------------------------------------------------------------ PTX helpers --
 

@@ -50,16 +50,16 @@ static __device__ __noinline__ void d_walk(const MatchParams *PP, uint64_t ri) {
 // lane, when its part is full.
 __device__ __forceinline__ void d_flush(const MatchParams &P, const uint32_t *pend, uint32_t n,
                                         uint32_t gw, uint32_t gstride, uint32_t lane) {
-    const uint32_t sub = gw & P.wsub_mask;
+    const uint32_t sub = chk32(P, gw & P.wsub_mask, WSUB_MAX);
     uint32_t *cnt = P.wcnt + sub * WSUB_STRIDE;
     uint64_t *buf = P.wbuf + (size_t)sub * P.wsub_cap;
     uint32_t base = P.wsub_cap;
     if (lane == 0 && *(volatile uint32_t *)cnt < P.wsub_cap) base = atomicAdd(cnt, n);
     base = __shfl_sync(0xFFFFFFFFu, base, 0);
     for (uint32_t e = lane; e < n; e += 32) {
-        const uint32_t v = pend[e];
+        const uint32_t v = pend[chk32(P, e, DQCAP)];
         const uint64_t u = ((gw + (uint64_t)(v >> 10) * gstride) << 1) + ((v >> 9) & 1u);
-        const uint64_t ri = (u << SLICE_SHIFT) + (v & (SLICE - 1));
+        const uint64_t ri = chk(P, (u << SLICE_SHIFT) + (v & (SLICE - 1)), (uint64_t)P.n_tiles << SLICE_SHIFT);
         if (base + e < P.wsub_cap) buf[base + e] = ri;
         else d_walk(&P, ri);
     }
@@ -114,8 +114,9 @@ __global__ void __launch_bounds__(DNW * 32, 1) k_scand(const __grid_constant__ M
     const uint8_t *src = P.in + ((uint64_t)gw << (SLICE_SHIFT + 1)) + lane * 32u;
     auto load = [&](uint32_t i, WChunk &c, uint4 &h) {
         if (i < n_ok) {
-            w_load32(src, al32, c);
-            h = ld_stream16_if(l31, src + 32);
+            const uint8_t *s = chk_in(P, src, l31 ? 48 : 32);
+            w_load32(s, al32, c);
+            h = ld_stream16_if(l31, s + 32);
             return;
         }
         const uint64_t s0 = (gw + (uint64_t)i * gstride) << (SLICE_SHIFT + 1), o = s0 + lane * 32u;
@@ -184,7 +185,7 @@ __global__ void __launch_bounds__(DNW * 32, 1) k_scand(const __grid_constant__ M
             mm &= mm - 1;
             const uint32_t lo = j < 16 ? w0 : w1, hi = j < 16 ? w1 : w2;
             const uint32_t t = __funnelshift_r(lo, hi, 2 * (j & 15)) & ((1u << (2 * D_LIST_SYMS)) - 1u);
-            A.list[at++] = (lane * 32 + j) | (t << 10) | (((root >> j) & 1u) ? D_LIST_ROOT : 0u);
+            A.list[chk32(P, at++, 2 * SLICE)] = (lane * 32 + j) | (t << 10) | (((root >> j) & 1u) ? D_LIST_ROOT : 0u);
         }
         __syncwarp();
         // the records of both slices, 32 candidates at a time (no candidate of
@@ -197,7 +198,7 @@ __global__ void __launch_bounds__(DNW * 32, 1) k_scand(const __grid_constant__ M
             const bool second = idx >= tot_a;
             const uint32_t slot = second ? idx - tot_a : idx;
             if (idx < tot) {
-                const uint32_t e = A.list[idx];
+                const uint32_t e = A.list[chk32(P, idx, 2 * SLICE)];
                 const uint64_t u = u0 + (second ? 1 : 0);
                 uint32_t fin, keys = 0;
                 if (e & D_LIST_ROOT) {
@@ -208,12 +209,12 @@ __global__ void __launch_bounds__(DNW * 32, 1) k_scand(const __grid_constant__ M
                     const uint32_t x = t & kmask;
                     const uint32_t r = (uint32_t)chk(
                         P, prefix_rank(Fs + (rep ? copy : 0u), rep, Cs, P.c_shift, x), P.T.n_e[k]);
-                    const uint32_t ev = ES ? Es[r] : __ldg(P.E + r);
+                    const uint32_t ev = ES ? Es[chk32(P, r, P.tbl_e_words)] : __ldg(P.E + r);
                     if (ev & D_CONT) {
                         pend = true;
                         if (masks) {
                             // four mask bits an entry (all: it reports output)
-                            const uint32_t mr = (Ms[r >> 3] >> (4 * (r & 7))) & 15u;
+                            const uint32_t mr = (Ms[chk32(P, r >> 3, P.tbl_m_words)] >> (4 * (r & 7))) & 15u;
                             const uint32_t c = (t >> (2 * k)) & 3u;
                             pend = mr == 15u || (c < sigma && ((mr >> c) & 1u));
                         }
@@ -223,17 +224,17 @@ __global__ void __launch_bounds__(DNW * 32, 1) k_scand(const __grid_constant__ M
                         // the others stays in 32 bits)
                         fin = ev;
                         if ((ev & FIN_LEN_ESC) != FIN_LEN_ESC) keys = ev & FIN_LEN_ESC;
-                        else atomicAdd((unsigned long long *)(P.tile_k + u),
+                        else atomicAdd((unsigned long long *)(P.tile_k + chk(P, u, P.n_tiles)),
                                        (unsigned long long)fin_len_c(P, ev));
                     }
                 }
                 keys_a += second ? 0u : keys;
                 keys_b += second ? keys : 0u;
-                P.recs[(size_t)u * P.unit_cap + slot] = ((uint64_t)(e & (SLICE - 1)) << 32) | fin;
+                P.recs[chk(P, (size_t)u * P.unit_cap + slot, (uint64_t)P.n_tiles * P.unit_cap)] = ((uint64_t)(e & (SLICE - 1)) << 32) | fin;
             }
             const uint32_t pm = __ballot_sync(0xFFFFFFFFu, pend);
             if (pm) {
-                if (pend) A.pend[np + __popc(pm & lt)] = (i << 10) | (second ? (uint32_t)SLICE : 0u) | slot;
+                if (pend) A.pend[chk32(P, np + __popc(pm & lt), DQCAP)] = (i << 10) | (second ? (uint32_t)SLICE : 0u) | slot;
                 np += __popc(pm);
                 if (np > DQCAP - 32) {
                     __syncwarp();
@@ -247,8 +248,9 @@ __global__ void __launch_bounds__(DNW * 32, 1) k_scand(const __grid_constant__ M
         if (lane < 2) {
             const uint32_t n = lane ? tot - tot_a : tot_a;
             if (n) {
-                P.tile_m[u0 + lane] = n;
-                atomicAdd((unsigned long long *)(P.tile_k + u0 + lane),
+                const uint64_t u = chk(P, u0 + lane, P.n_tiles);
+                P.tile_m[u] = n;
+                atomicAdd((unsigned long long *)(P.tile_k + u),
                           (unsigned long long)(lane ? keys_b : keys_a));
             }
         }

@@ -92,16 +92,16 @@ struct WConst {
 
 // Bit 0 of the result: whether the window at symbol j of the lane passes.
 template <int PACKED, int NB, int G5, int TB>
-__device__ __forceinline__ uint32_t w_lookup(const uint32_t (&w)[9], int j, const WConst &K) {
+__device__ __forceinline__ uint32_t w_lookup(const MatchParams &P, const uint32_t (&w)[9], int j, const WConst &K) {
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t t = w_twin<PACKED>(w, j);
     uint32_t y = t * K.gm;
     if (G5) y += w_twin<PACKED>(w, j + 1) * WIN_MUL2;
     const uint32_t h = __umulhi(y, K.hm);
     uint32_t x;
-    if (TB == WT_L2) x = __ldg(K.tbl + h);
-    else if (TB == WT_ONE) x = reinterpret_cast<const uint32_t *>(smem)[h];
-    else x = *reinterpret_cast<const uint32_t *>(smem + ((h & K.amask) | K.c4));
+    if (TB == WT_L2) x = __ldg(K.tbl + chk32(P, h, P.w_words));
+    else if (TB == WT_ONE) x = reinterpret_cast<const uint32_t *>(smem)[chk32(P, h, P.w_words)];
+    else x = *reinterpret_cast<const uint32_t *>(smem + chk32(P, (h & K.amask) | K.c4, (4ull * P.w_words) << P.w_rep));
     uint32_t r = __funnelshift_r(x, x, w_twin<PACKED>(w, j + (PACKED ? 0 : 2)));
     if (NB >= 2) r &= __funnelshift_r(x, x, w_twin<PACKED>(w, j + (PACKED ? 3 : 0)));
     if (NB >= 3) r &= __funnelshift_r(x, x, w_twin<PACKED>(w, j + (PACKED ? 6 : 1)));
@@ -111,7 +111,7 @@ __device__ __forceinline__ uint32_t w_lookup(const uint32_t (&w)[9], int j, cons
 // All windows of the lane's 32 positions: bit i is set when the one at
 // symbol i * S + S - 1 passes.
 template <int PACKED, int S, int NB, int G5, int TB>
-__device__ __forceinline__ uint32_t w_filter(const uint32_t (&w)[9], const WConst &K) {
+__device__ __forceinline__ uint32_t w_filter(const MatchParams &P, const uint32_t (&w)[9], const WConst &K) {
     constexpr int NWIN = 32 / S;
     if constexpr (NWIN >= 8) {
         // each test's bit is shifted in at the top of a word: chains of eight
@@ -123,7 +123,7 @@ __device__ __forceinline__ uint32_t w_filter(const uint32_t (&w)[9], const WCons
 #pragma unroll
             for (int c = 0; c < NWIN / 8; c++)
                 acc[c] = __funnelshift_r(
-                    acc[c], w_lookup<PACKED, NB, G5, TB>(w, (8 * c + i) * S + S - 1, K), 1);
+                    acc[c], w_lookup<PACKED, NB, G5, TB>(P, w, (8 * c + i) * S + S - 1, K), 1);
         // bits 24..31 of each chain
         if (NWIN == 8) return acc[0] >> 24;
         if constexpr (NWIN == 16) return __byte_perm(acc[0], acc[1], 0x0073) & 0xFFFFu;
@@ -134,7 +134,7 @@ __device__ __forceinline__ uint32_t w_filter(const uint32_t (&w)[9], const WCons
         uint32_t m = 0;
 #pragma unroll
         for (int i = 0; i < NWIN; i++)
-            m |= (w_lookup<PACKED, NB, G5, TB>(w, i * S + S - 1, K) & 1u) << i;
+            m |= (w_lookup<PACKED, NB, G5, TB>(P, w, i * S + S - 1, K) & 1u) << i;
         return m;
     }
 }
@@ -198,7 +198,7 @@ __device__ __forceinline__ uint32_t w_limit(const MatchParams &P, uint32_t u, ui
     uint32_t lo = 1, hi = P.n_seg;
     if (INDEXED) {
         // (bounded: offsets out of order leave some indices unwritten)
-        lo = __ldg(P.unit_seg + u);
+        lo = __ldg(P.unit_seg + chk32(P, u, P.n_tiles));
         hi = u + 1 < P.n_tiles ? __ldg(P.unit_seg + u + 1) : P.n_seg;
         lo = lo < P.n_seg ? lo : P.n_seg;
         hi = hi < P.n_seg ? hi : P.n_seg;
@@ -330,7 +330,7 @@ __device__ __forceinline__ void w_flush(const MatchParams &P, const uint32_t *q,
         for (int r = 0; r < R; r++) {
             const uint32_t e = e0 + 32 * r + lane;
             const bool in = e < n * S;
-            const uint32_t v = q[in ? e / S : 0u];
+            const uint32_t v = q[in ? chk32(P, e / S, WQCAP) : 0u];
             const uint64_t pr = gw + (uint64_t)(v >> 10) * gstride;
             const uint64_t p = (pr << (SLICE_SHIFT + 1)) + (v & 1023u) - (S - 1 - e % S);
             const bool on = in && p < P.starts_end;
@@ -354,7 +354,7 @@ __device__ __forceinline__ void w_flush(const MatchParams &P, const uint32_t *q,
         if (tot == 0) continue;
         // the warp's part of the buffer; no reservation once it is full, so
         // that its counter stays within one reservation per warp of its size
-        const uint32_t sub = gw & P.wsub_mask;
+        const uint32_t sub = chk32(P, gw & P.wsub_mask, WSUB_MAX);
         uint32_t *cnt = P.wcnt + sub * WSUB_STRIDE;
         uint64_t *buf = P.wbuf + (size_t)sub * P.wsub_cap;
         uint32_t base = P.wsub_cap;
@@ -470,8 +470,9 @@ __global__ void __launch_bounds__((TB == WT_L2 ? WNW_SMALL : WNW) * 32, 1)
     // past the clean ones as far as the input goes in whole 16-byte pieces
     auto load = [&](uint32_t i, WChunk &c, uint4 &h) {
         if (i < n_ok) {
-            w_load32(src, al32, c);
-            h = load_head(l31, src + 32);
+            const uint8_t *s = chk_in(P, src, l31 ? 32 + HALO : 32);
+            w_load32(s, al32, c);
+            h = load_head(l31, s + 32);
             return;
         }
         const uint64_t s0 = (gw + (uint64_t)i * gstride) << (SLICE_SHIFT + 1), o = s0 + lane * 32u;
@@ -507,7 +508,7 @@ __global__ void __launch_bounds__((TB == WT_L2 ? WNW_SMALL : WNW) * 32, 1)
 #pragma unroll
                 for (int x = 3; x < 9; x++) w[x] = 0;
             }
-            m = w_filter<PACKED, S, NB, G5, TB>(w, K);
+            m = w_filter<PACKED, S, NB, G5, TB>(P, w, K);
             if (P.w_badmask) {
                 // bytes outside the packed symbol range, where H would need
                 // completions over them (patterns that end inside a window):
@@ -540,7 +541,7 @@ __global__ void __launch_bounds__((TB == WT_L2 ? WNW_SMALL : WNW) * 32, 1)
             if (m) {
                 const uint32_t j = __ffs(m) - 1;
                 m &= m - 1;
-                q[qn + __popc(any & lt)] = (i << 10) + (lane * 32 + j * S + S - 1);
+                q[chk32(P, qn + __popc(any & lt), WQCAP)] = (i << 10) + (lane * 32 + j * S + S - 1);
             }
             qn += __popc(any);
             if (qn > WQCAP - 32 || i >= n_it) {
@@ -647,7 +648,7 @@ __global__ void __launch_bounds__(RES_WARPS * 32, RES_CTAS)
             state[u] = on ? 0 : -1;
             st[u] = 0;
             if (DENSE) {
-                const uint64_t r = on ? P.recs[v] : 0ull;
+                const uint64_t r = on ? P.recs[chk(P, v, (uint64_t)P.n_tiles << SLICE_SHIFT)] : 0ull;
                 unit[u] = (uint32_t)chk(P, v >> SLICE_SHIFT, P.n_tiles ? P.n_tiles : 1);
                 slot[u] = (uint32_t)v & (SLICE - 1);
                 pos[u] = (uint32_t)(r >> 32);
@@ -766,7 +767,7 @@ __global__ void __launch_bounds__(RES_WARPS * 32, RES_CTAS)
             const bool w = state[u] == 0;
             const uint32_t bm = __ballot_sync(0xFFFFFFFFu, w);
             if (w) {
-                const uint32_t t = nt + __popc(bm & lt);
+                const uint32_t t = chk32(P, nt + __popc(bm & lt), WRB);
                 T.unit[t] = unit[u];
                 T.pos[t] = pos[u];
                 T.q[t] = q[u];
