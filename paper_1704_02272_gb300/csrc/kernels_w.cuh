@@ -147,40 +147,28 @@ __device__ __forceinline__ uint32_t w_filter(const MatchParams &P, const uint32_
 // matches would queue on one chunk's word (1 GiB of packets: 0.8 instead of
 // 0.36 ms), and k_reduce sums them.
 //
-// SHARED: calling lanes whose matches lie in one slice add once.  For the
-// scan's own walks, where most starts may match: 32 adds then queued on one
-// word (8 MiB of one symbol that two patterns repeat, all / shared: 1,079 /
-// 610 us a call).  Not for the resolver, whose few matches lie apart: shared
-// there too, 1 GiB of packets 1,204 -> 1,222 us, and by slices told apart with
-// a match instruction 1,249.
+// SHARED: the calling lanes' matches of one slice add once.  For the scan's own
+// walks, where most starts may match: 32 adds then queued on one word (8 MiB of
+// one symbol that two patterns repeat, apart / shared: 1,074 / 630 us a call; 9
+// MB of printable packets against 50,000 signatures 319 / 309).  Not for the
+// resolver, whose few matches lie apart: shared there too, 1 GiB of packets
+// 1,204 -> 1,249 us.
 template <bool SHARED>
 __device__ __forceinline__ void w_emit(const MatchParams &P, uint32_t u, uint32_t pos, uint32_t fin) {
     u = (uint32_t)chk(P, u, P.n_tiles);
-    const uint32_t cap = P.unit_cap;
+    const uint32_t cap = P.unit_cap, lane = threadIdx.x & 31;
+    const uint32_t same = SHARED ? __match_any_sync(__activemask(), u) : 1u << lane;
+    const uint32_t first = __ffs(same) - 1;
     unsigned long long keys = fin_len_c(P, fin);
-    uint32_t n = 1, lower = 0;  // matches of this add, and those before the lane's
-    uint32_t act = 0, first = 0;
-    bool one = false, adds = true;
-    if (SHARED) {
-        act = __activemask();
-        first = __ffs(act) - 1;
-        one = __all_sync(act, u == __shfl_sync(act, u, first));
-        if (one) {
-            // (lists of at most 2^24 ids: a warp's fit 32 bits)
-            keys = __reduce_add_sync(act, (uint32_t)keys);
-            n = __popc(act);
-            const uint32_t lane = threadIdx.x & 31;
-            lower = __popc(act & ((1u << lane) - 1u));
-            adds = lane == first;
-        }
-    }
+    if (SHARED) keys = __reduce_add_sync(same, (uint32_t)keys);  // (lists of at most 2^24 ids)
     uint32_t rank = 0;
-    if (adds) {
-        rank = (uint32_t)(atomicAdd((unsigned long long *)(P.tile_k + u),
-                                    ((unsigned long long)n << UNIT_KEY_BITS) | keys) >> UNIT_KEY_BITS);
+    if (!SHARED || lane == first) {
+        const unsigned long long n = SHARED ? __popc(same) : 1;
+        rank = (uint32_t)(atomicAdd((unsigned long long *)(P.tile_k + u), (n << UNIT_KEY_BITS) | keys) >>
+                          UNIT_KEY_BITS);
         if (P.chunk_adds) atomicAdd((unsigned long long *)(P.chunk + (u >> P.chunk_shift)), keys);
     }
-    if (SHARED && one) rank = __shfl_sync(act, rank, first) + lower;
+    if (SHARED) rank = __shfl_sync(same, rank, first) + __popc(same & ((1u << lane) - 1u));
     if (rank < cap) P.recs[(size_t)u * cap + rank] = ((uint64_t)pos << 32) | fin;
 }
 
