@@ -41,7 +41,7 @@ static __device__ __noinline__ void d_walk(const MatchParams *PP, uint64_t ri) {
     const MatchParams &P = *PP;
     const uint64_t u = ri >> SLICE_SHIFT, rec = P.recs[ri];
     const uint32_t pos = (uint32_t)(rec >> 32);
-    const uint32_t fin = w_walk_any(P, u << SLICE_SHIFT, pos, w_limit<false>(P, (uint32_t)u, (u << SLICE_SHIFT) + pos));
+    const uint32_t fin = w_walk_any(P, u << SLICE_SHIFT, pos, w_limit(P, (uint32_t)u, (u << SLICE_SHIFT) + pos));
     P.recs[ri] = ((uint64_t)pos << 32) | fin;
     if (fin) atomicAdd((unsigned long long *)(P.tile_k + u), (unsigned long long)fin_len_c(P, fin));
 }

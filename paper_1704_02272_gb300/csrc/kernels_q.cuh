@@ -606,36 +606,41 @@ __device__ __forceinline__ void filter_slice(const MatchParams &P, const uint8_t
 // with few, each lane finds its unit's index by binary search over them.
 // (1.36 million packets in 1 GiB: the search alone took 51 us.)  Offsets that
 // are not in order may leave units unwritten: readers bound what they find.
+// The indices are for later launches alone: any warp writes any unit's.  CHECK,
+// WRITE: only the one or the other, where two launches share the work.
+template <bool CHECK, bool WRITE>
 __device__ __forceinline__ void unit_segments(const MatchParams &P, uint32_t gw, uint32_t nw,
                                               uint32_t lane) {
     const uint64_t *seg = P.seg;
     const uint32_t n_seg = P.n_seg, n = P.n_tiles;
-    if (gw == 0 && lane == 0 && (__ldg(seg) != 0 || __ldg(seg + n_seg) != P.n))
+    if (CHECK && gw == 0 && lane == 0 && (__ldg(seg) != 0 || __ldg(seg + n_seg) != P.n))
         atomicOr(&P.hdr->status, ST_BADSEG);
     const bool many = n_seg >= n / 8;
-    for (uint64_t s0 = (uint64_t)gw * 32; s0 < n_seg; s0 += (uint64_t)nw * 32) {
-        const uint64_t s = s0 + lane;
-        uint64_t a = 0, b = 0;  // units that start in segment s: [a, b)
-        if (s < n_seg) {
-            const uint64_t o0 = __ldg(seg + s), o1 = __ldg(seg + s + 1);
-            if (o1 < o0) atomicOr(&P.hdr->status, ST_BADSEG);
-            a = (o0 + SLICE - 1) >> SLICE_SHIFT;
-            b = (o1 + SLICE - 1) >> SLICE_SHIFT;
-            if (b > n) b = n;
-        }
-        if (!many) continue;
-        const bool is_long = b > a && b - a > 16;
-        if (!is_long)
-            for (uint64_t u = a; u < b; u++) P.unit_seg[u] = (uint32_t)s + 1;
-        uint32_t m = __ballot_sync(0xFFFFFFFFu, is_long);
-        while (m) {
-            const uint32_t j = __ffs(m) - 1;
-            m &= m - 1;
-            const uint64_t aj = __shfl_sync(0xFFFFFFFFu, a, j), bj = __shfl_sync(0xFFFFFFFFu, b, j);
-            for (uint64_t u = aj + lane; u < bj; u += 32) P.unit_seg[u] = (uint32_t)s0 + j + 1;
+    if (CHECK || many) {
+        for (uint64_t s0 = (uint64_t)gw * 32; s0 < n_seg; s0 += (uint64_t)nw * 32) {
+            const uint64_t s = s0 + lane;
+            uint64_t a = 0, b = 0;  // units that start in segment s: [a, b)
+            if (s < n_seg) {
+                const uint64_t o0 = __ldg(seg + s), o1 = __ldg(seg + s + 1);
+                if (CHECK && o1 < o0) atomicOr(&P.hdr->status, ST_BADSEG);
+                a = (o0 + SLICE - 1) >> SLICE_SHIFT;
+                b = (o1 + SLICE - 1) >> SLICE_SHIFT;
+                if (b > n) b = n;
+            }
+            if (!WRITE || !many) continue;
+            const bool is_long = b > a && b - a > 16;
+            if (!is_long)
+                for (uint64_t u = a; u < b; u++) P.unit_seg[u] = (uint32_t)s + 1;
+            uint32_t m = __ballot_sync(0xFFFFFFFFu, is_long);
+            while (m) {
+                const uint32_t j = __ffs(m) - 1;
+                m &= m - 1;
+                const uint64_t aj = __shfl_sync(0xFFFFFFFFu, a, j), bj = __shfl_sync(0xFFFFFFFFu, b, j);
+                for (uint64_t u = aj + lane; u < bj; u += 32) P.unit_seg[u] = (uint32_t)s0 + j + 1;
+            }
         }
     }
-    if (many) return;
+    if (!WRITE || many) return;
     for (uint64_t u = (uint64_t)gw * 32 + lane; u < n; u += (uint64_t)nw * 32) {
         const uint64_t start = u << SLICE_SHIFT;
         uint32_t lo = 1, hi = n_seg;

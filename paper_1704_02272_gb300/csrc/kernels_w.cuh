@@ -174,23 +174,17 @@ __device__ __forceinline__ void w_emit(const MatchParams &P, uint32_t u, uint32_
 
 // Walk limit of start p of slice u, relative to the slice start: the first
 // offset above p, found between the slice's first offset index and the next
-// slice's (INDEXED), or among all offsets.  The indices are written by the
-// scan launch itself, each by any of its warps, so that only the launches
-// after it may read them.
-template <bool INDEXED>
+// slice's (both written by the launch before the scan).
 __device__ __forceinline__ uint32_t w_limit(const MatchParams &P, uint32_t u, uint64_t p) {
     const uint64_t ustart = (uint64_t)u << SLICE_SHIFT;
     const uint64_t remain = P.n - ustart;
     const uint32_t rem = remain < LIM_MAX ? (uint32_t)remain : LIM_MAX;
     if (P.n_seg <= 1) return rem;
-    uint32_t lo = 1, hi = P.n_seg;
-    if (INDEXED) {
-        // (bounded: offsets out of order leave some indices unwritten)
-        lo = __ldg(P.unit_seg + chk32(P, u, P.n_tiles));
-        hi = u + 1 < P.n_tiles ? __ldg(P.unit_seg + u + 1) : P.n_seg;
-        lo = lo < P.n_seg ? lo : P.n_seg;
-        hi = hi < P.n_seg ? hi : P.n_seg;
-    }
+    // (bounded: offsets out of order leave some indices unwritten)
+    uint32_t lo = __ldg(P.unit_seg + chk32(P, u, P.n_tiles));
+    uint32_t hi = u + 1 < P.n_tiles ? __ldg(P.unit_seg + u + 1) : P.n_seg;
+    lo = lo < P.n_seg ? lo : P.n_seg;
+    hi = hi < P.n_seg ? hi : P.n_seg;
     while (lo < hi) {
         const uint32_t mid = (lo + hi) >> 1;
         if (__ldg(P.seg + mid) > p) hi = mid; else lo = mid + 1;
@@ -233,7 +227,7 @@ __device__ __forceinline__ uint32_t w_walk_any(const MatchParams &P, uint64_t ub
 static __device__ __noinline__ void w_walk(const MatchParams *PP, uint64_t p) {
     const MatchParams &P = *PP;
     const uint32_t u = (uint32_t)(p >> SLICE_SHIFT), pos = (uint32_t)p & (SLICE - 1);
-    const uint32_t fin = w_walk_any(P, (uint64_t)u << SLICE_SHIFT, pos, w_limit<false>(P, u, p));
+    const uint32_t fin = w_walk_any(P, (uint64_t)u << SLICE_SHIFT, pos, w_limit(P, u, p));
     if (fin) w_emit<true>(P, u, pos, fin);
 }
 
@@ -430,7 +424,6 @@ __global__ void __launch_bounds__((TB == WT_L2 ? WNW_SMALL : WNW) * 32, 1)
     }
     // from here on the call's counters are used, zeroed by the kernel before
     dep_wait();
-    if (P.n_seg > 1) unit_segments(P, gw, gstride, lane);
     WConst K;
     K.gm = P.w_gm;
     K.tbl = P.T.H;
@@ -823,6 +816,9 @@ __global__ void __launch_bounds__(RES_WARPS * 32, RES_CTAS)
         }
         __syncwarp();
     }
+    // the offsets are checked here, by the last warps first: they have the
+    // fewest entries
+    if (!DENSE && P.n_seg > 1) unit_segments<true, false>(P, gs - 1 - gw, gs, lane);
 }
 
 }  // namespace pfac

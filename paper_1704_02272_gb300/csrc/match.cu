@@ -129,10 +129,11 @@ __global__ void k_bounds(const MatchParams P) {
     }
 }
 
-// The segment data of the slice kernels (the window kernel does this itself).
+// The segment data of the slice kernels (the window kernel's: k_zero and
+// k_wresolve).
 __global__ void k_unitseg(const MatchParams P) {
     const uint32_t gt = blockIdx.x * blockDim.x + threadIdx.x;
-    unit_segments(P, gt >> 5, (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
+    unit_segments<true, true>(P, gt >> 5, (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
 }
 
 // ------------------------------------------------ key-count scan ----------
@@ -165,11 +166,18 @@ __device__ __forceinline__ uint64_t block_excl_scan(uint64_t v, uint64_t *sh, ui
     return r;
 }
 
-// Zeroes the head of the workspace (n 16-byte words): a kernel rather than a
-// memset, so that the scan's table fill overlaps it.
-__global__ void __launch_bounds__(256) k_zero(uint4 *p, uint64_t n) {
-    for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256)
-        p[i] = make_uint4(0, 0, 0, 0);
+// Zeroes the head of the workspace (n 16-byte words) and writes the slices'
+// first offset indices, which the scan reads where it walks starts itself: a
+// kernel rather than a memset, so that the scan's table fill overlaps it.  (The
+// resolver checks the offsets: the status is among what is zeroed here.)  With
+// the indices written by the scan launch, its own walks could not use them and
+// searched all offsets: a request of 9 MB against 50,000 signatures, a fifth of
+// whose starts are walked there, 74 us, with them 63; printable text 309 and
+// 270.
+__global__ void __launch_bounds__(256) k_zero(const __grid_constant__ MatchParams P, uint4 *p, uint64_t n) {
+    const uint64_t t = (uint64_t)blockIdx.x * 256 + threadIdx.x, nt = (uint64_t)gridDim.x * 256;
+    for (uint64_t i = t; i < n; i += nt) p[i] = make_uint4(0, 0, 0, 0);
+    if (P.n_seg > 1) unit_segments<false, true>(P, (uint32_t)(t >> 5), (uint32_t)(nt >> 5), threadIdx.x & 31);
 }
 
 // Key counts of the chunks of units, where they are not added up as matches
@@ -242,7 +250,7 @@ static __device__ __noinline__ void expand_unit(const MatchParams *PP, uint64_t 
         const uint32_t pos = p0 + lane;
         uint32_t fin = 0, L = 0;
         if (us + pos < P.starts_end) {
-            fin = w_walk_any(P, us, pos, w_limit<true>(P, (uint32_t)t, us + pos));
+            fin = w_walk_any(P, us, pos, w_limit(P, (uint32_t)t, us + pos));
             if (fin) L = fin_len_c(P, fin);
         }
         const uint32_t before = keys_before<32>(pos, L, false, lane);
@@ -1275,9 +1283,11 @@ extern "C" int pfac_match_async(const pfac_table *t, const uint8_t *d_input, uin
     if (ent) {
         uint4 *zp = (uint4 *)P.hdr;
         uint64_t zn = zero / 16;
-        void *args[] = {&zp, &zn};
-        const uint64_t zb = (zn + 1023) / 1024;
-        e = launch((const void *)k_zero, (uint32_t)std::min<uint64_t>(zb ? zb : 1, (uint64_t)nsm * 4), 256, args,
+        void *args[] = {&P, &zp, &zn};
+        // four words a thread, and one slice or offset
+        const uint64_t idx = n_segments > 1 ? std::max<uint64_t>(P.n_tiles, n_segments) : 0;
+        const uint64_t zb = std::max<uint64_t>((zn + 1023) / 1024, (idx + 255) / 256);
+        e = launch((const void *)k_zero, (uint32_t)std::min<uint64_t>(zb ? zb : 1, (uint64_t)nsm * 8), 256, args,
                    0, st, false);
     } else {
         e = cudaMemsetAsync(P.hdr, 0, zero, st);
