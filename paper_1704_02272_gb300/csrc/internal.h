@@ -46,6 +46,10 @@ void clear_error();
 // with another GPU's pointers.
 int check_table_device(const pfac_table *t, void *cuda_stream, const char *who);
 
+// Shared-memory wavefronts of one warp-wide load of random words with 2^i
+// copies interleaved over the banks: lanes that share a copy collide.
+constexpr double LOAD_WAVEFRONTS[6] = {3.7, 3.4, 3.1, 2.85, 2.0, 1.0};
+
 // Bytes of a workspace that do not grow with the input, at most: a fixed
 // scratch or pool of N bytes is made this much larger, so that it holds what
 // takes N bytes for its input alone.

@@ -413,7 +413,7 @@ enum { SCAN_QUEUED = PFAC_KERNEL_QUEUED, SCAN_REGISTER = PFAC_KERNEL_REGISTER, S
 struct WsLayout {
     uint64_t hdr, tile_m, tile_k, key_off, chunk, ovf, recs, bounds, defer, dbatch, total;
     uint64_t wbuf, wcnt;
-    uint32_t n_tiles, n_chunks, defer_cap, dbatch_cap, wsub_cap, wsubs;
+    uint32_t n_tiles, defer_cap, dbatch_cap, wsub_cap, wsubs;
 };
 
 // entries per slice the resolver kernel's buffer holds (more go to the
@@ -437,8 +437,6 @@ static WsLayout ws_layout(uint64_t n_bytes, uint32_t n_seg, const Plan &pl) {
     const uint64_t ub = 1ull << pl.unit_shift;
     const uint64_t nt = (n_bytes + ub - 1) / ub;
     L.n_tiles = (uint32_t)nt;
-    const uint32_t cs = chunk_shift(nt);
-    L.n_chunks = (uint32_t)((nt + (1ull << cs) - 1) >> cs);
     uint64_t o = 0;
     auto put = [&](uint64_t sz) {
         const uint64_t at = o;
@@ -446,8 +444,8 @@ static WsLayout ws_layout(uint64_t n_bytes, uint32_t n_seg, const Plan &pl) {
         return at;
     };
     L.hdr = put(sizeof(WsHeader));
-    // one memset zeroes the header and the counts (the record counts only
-    // where they are kept apart from the key counts)
+    // the call's first launch zeroes the header and the counts (the record
+    // counts only where they are kept apart from the key counts)
     L.wcnt = put(entries ? (uint64_t)WSUB_MAX * WSUB_STRIDE * 4 : 0);
     L.chunk = put((uint64_t)CHUNKS_MAX * 8);
     L.tile_k = put(nt * 8);
@@ -505,12 +503,7 @@ static size_t queued_smem(uint64_t words, uint32_t nw = QW) {
     return tbl + nw * sizeof(WarpArea);
 }
 
-// Shared-memory wavefronts of one warp-wide bitmap load with 2^rep copies
-// (interleaved word by word): lanes sharing a copy collide on a bank.
-static double load_wavefronts(int rep) {
-    static const double wf[6] = {3.7, 3.4, 3.1, 2.85, 2.0, 1.0};
-    return wf[rep < 0 ? 0 : (rep > 5 ? 5 : rep)];
-}
+static double load_wavefronts(int rep) { return LOAD_WAVEFRONTS[rep < 0 ? 0 : (rep > 5 ? 5 : rep)]; }
 
 // Estimated warp instructions per 512-byte slice of a first stage that
 // passes a share `dens` of the positions (measured orders of magnitude:

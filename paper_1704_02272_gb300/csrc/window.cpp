@@ -12,15 +12,12 @@
 
 #include <algorithm>
 
+#include "internal.h"
 #include "table.h"
 
 namespace pfac {
 
 namespace {
-
-// Shared-memory wavefronts of one warp-wide load of random words with 2^rep
-// copies interleaved over the banks.
-constexpr double WAVEFRONTS[6] = {3.7, 3.4, 3.1, 2.85, 2.0, 1.0};
 
 // Most strings inserted (completions of short patterns included).
 constexpr double MAX_STRINGS = 2.0e6;
@@ -133,7 +130,7 @@ bool build_window_filter(const std::vector<WinPat> &pats, uint32_t sigma, uint32
             const double L = 16.0 / s.S;
             const double alu = 16.0 + (packed ? 4.0 : 0.0) +
                                L * (8.0 + 2.0 * (s.nb - 1) + s.g5) / 4.0 * 1.2;
-            const double lds = L * WAVEFRONTS[rep] * 1.05;
+            const double lds = L * LOAD_WAVEFRONTS[rep] * 1.05;
             const double cand = 512.0 / s.S * pass;
             // starts left after the prefix bitmap
             const double left = 512.0 * match +
@@ -153,7 +150,6 @@ bool build_window_filter(const std::vector<WinPat> &pats, uint32_t sigma, uint32
                 out->glen = glen;
                 out->packed = packed;
                 out->shorts = min_len < glen + s.S - 1 ? 1u : 0u;
-                out->cost = cost;
             }
         }
     }

@@ -13,15 +13,12 @@ struct WinPat {
 
 struct WindowFilter {
     uint32_t words = 0, rep = 0, stride = 0, nb = 0, gw = 0, glen = 0, packed = 0, shorts = 0;
-    double cost = 0;  // estimated SM cycles per 512-byte slice, resolution included
     std::vector<uint32_t> H;
 };
 
 // Picks the filter with the least estimated cost for uniform text and builds
 // it; false when none is estimated to pay.  dens_f: share of uniform windows
-// that pass the prefix bitmap the scan tests candidates against; real: share
-// of starts whose walk reaches the depth of that bitmap's table or reports
-// something there.
+// that pass the prefix bitmap the scan tests candidates against.
 bool build_window_filter(const std::vector<WinPat> &pats, uint32_t sigma, uint32_t bps, double dens_f,
                          WindowFilter *out);
 
