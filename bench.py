@@ -40,29 +40,15 @@ sys.path.insert(0, ROOT)
 
 import workloads  # noqa: E402
 
-# dram__bytes_read.sum + dram__bytes_write.sum of one scan launch from ncu
-# captures (summaries under profiles/), per workload and scan plan (the
-# autotuner settles on one of near-equal plans), with the digest of the
-# kernel sources they were taken on; reported only while the sources match
+# dram__bytes_read.sum + dram__bytes_write.sum of one call's scan launches (the
+# scan kernel and its resolver) from ncu captures (summaries under profiles/),
+# per workload and the kernel and plan that ran, with the digest of the kernel
+# sources they were taken on; reported only while the sources match
 MEASURED_TRAFFIC = {
-    "dna": [(310759680, "d100e0d9e6ba3865",
-             {"variant": 1, "prefix_depth": 10, "bitmap_copies": 1, "child_masks": 1,
-              "gram_filter": 1, "prefix_bytes": 1, "warps_per_cta": 16, "scan_kernel": 1,
-              "records_per_slice": 512, "resolver": 2}),
-            (311110912, "d100e0d9e6ba3865",
-             {"variant": 1, "prefix_depth": 10, "bitmap_copies": 1, "child_masks": 1,
-              "gram_filter": 1, "prefix_bytes": 1, "warps_per_cta": 16, "scan_kernel": 1,
-              "records_per_slice": 32, "resolver": 2})],
-    "sweep-256-1000": [(550563584, "d100e0d9e6ba3865",
-                        {"variant": 1, "prefix_depth": 2, "bitmap_copies": 1, "child_masks": 1,
-                         "gram_filter": 2, "prefix_bytes": 1, "warps_per_cta": 16,
-                         "scan_kernel": 2, "records_per_slice": 32, "resolver": 2}),
-                       (553913344, "d100e0d9e6ba3865",
-                        {"variant": 2, "prefix_depth": 2, "bitmap_copies": 1, "child_masks": 2,
-                         "gram_filter": 2, "prefix_bytes": 1, "warps_per_cta": 16,
-                         "scan_kernel": 2, "records_per_slice": 32, "resolver": 1})],
+    "dna": [(506785280, "9b54e7b866d7831c", {"kernel_run": "window"})],
+    "sweep-256-1000": [(608744192, "9b54e7b866d7831c", {"kernel_run": "window"})],
 }
-KERNEL_SOURCES = ["kernels_q.cuh", "kernels_r.cuh", "kernels.cuh", "table.h"]
+KERNEL_SOURCES = ["kernels_d.cuh", "kernels_q.cuh", "kernels_r.cuh", "kernels_w.cuh", "kernels.cuh", "table.h"]
 SCAN_NAMES = {
     "window": "k_scanw with k_wresolve (compressed-table scan and its resolver)",
     "dense": "k_scand with k_wresolve (compressed-table scan and its resolver)",
@@ -447,7 +433,7 @@ def time_cell(pfac, torch, w, dev, stream, args, user_opt, workload_name, graph_
                 "unit": "GB/s", "frac": round(achieved / hbm_peak, 4),
                 "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)",
                 "traffic": args.traffic if (args.traffic is not None and graph_steps) else (
-                    measured_traffic(workload_name, plan) if not user_opt else None),
+                    measured_traffic(workload_name, dict(plan, kernel_run=route)) if not user_opt else None),
                 "kernel": SCAN_NAMES[route],
                 "alg_bytes_per_launch": alg_bytes,
                 "scan_pass_ms": round(scan_avg_ms, 4), "emit_pass_ms": round(emit_avg_ms, 4)}

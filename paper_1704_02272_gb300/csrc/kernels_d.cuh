@@ -21,7 +21,7 @@
 // its queue through L2, took 760 us; this one 162 us, and 43 us for the pending
 // records (206 us when each slice listed its candidates by itself, with half
 // the lanes idle).  It is bound by the instructions per position and per
-// candidate (68% issue, 70% of the ALU pipe at 206 us).
+// candidate (74% issue, 76% of the ALU pipe).
 #pragma once
 #include "kernels_w.cuh"
 
