@@ -1,7 +1,7 @@
 """GPU parity of the window kernel where its entry buffer is full and the text
-has many segments: walks inside the scan take their segment ends from the
-offsets alone, so neither what the workspace held before nor another call on
-the GPU changes a result.  The oracle's whole list is the reference."""
+has many segments: walks inside the scan take their segment ends from what the
+launch before wrote, so neither what the workspace held nor another call on the
+GPU changes a result.  The oracle's whole list is the reference."""
 import numpy as np
 import pytest
 import torch
